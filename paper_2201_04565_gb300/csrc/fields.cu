@@ -17,6 +17,7 @@
 #include <cmath>
 #include <vector>
 
+#include "exact64.cuh"
 #include "lsm_internal.h"
 
 namespace lsm {
@@ -67,15 +68,13 @@ k_fields(int64_t n, const int64_t *__restrict__ row, const uint32_t *__restrict_
             double d[DIM];
 #pragma unroll
             for (int c = 0; c < DIM; c++) d[c] = sub_(x[c * n + j], x[c * n + i]);
-            double r2 = add_(mul_(d[0], d[0]), mul_(d[1], d[1]));
-            if (DIM == 3) r2 = add_(r2, mul_(d[DIM - 1], d[DIM - 1]));
-            const double r = __dsqrt_rn(r2);
-            const double cs = div_(mul_(t.k, sub_(r, t.r0)), r);
+            double r2, st, f[DIM];
+            e64_force<DIM>(d, t.k, t.r0, r2, st, f);
 #pragma unroll
             for (int q = 0; q < NQ; q++) {
                 int a, b;
                 comp_pair(DIM, q, a, b);
-                S[q] = add_(S[q], mul_(0.5, mul_(d[a], mul_(cs, d[b]))));
+                S[q] = add_(S[q], mul_(0.5, mul_(d[a], f[b])));
             }
         }
         const double mp = mass[p];

@@ -26,6 +26,7 @@
 #include <cstdio>
 
 #include "dfloat.cuh"
+#include "exact64.cuh"
 #include "lsm_internal.h"
 
 namespace lsm {
@@ -39,7 +40,6 @@ constexpr int RED_THREADS = 1024;
 __device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sb(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double ml(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double dv(double a, double b) { return __ddiv_rn(a, b); }
 
 // Fixed-order block sum of one value per thread (TPB threads): warp xor tree,
 // then the warps in order. Deterministic for a given TPB.
@@ -88,16 +88,15 @@ k_springs(int64_t m, int64_t n, const int32_t *__restrict__ si, const int32_t *_
         double d[DIM];
 #pragma unroll
         for (int c = 0; c < DIM; c++) d[c] = sb(x[c * n + j], x[c * n + i]);
-        double r2;
+        double r2, e, f[DIM];  // EXACT64: e = r - r0, f the force on i
         if constexpr (PREC == LSM_PREC_EXACT64) {
-            r2 = ad(ml(d[0], d[0]), ml(d[1], d[1]));
-            if constexpr (DIM == 3) r2 = ad(r2, ml(d[2], d[2]));
+            e64_force<DIM>(d, t.k, t.r0, r2, e, f);
         } else {
             r2 = d[0] * d[0];
 #pragma unroll
             for (int c = 1; c < DIM; c++) r2 = fma(d[c], d[c], r2);
         }
-        if (BREAK && r2 > t.rc2) {
+        if (BREAK && e64_gt(r2, t.rc2)) {
             // Heaviside switch: the spring is broken for good and gives no
             // force from this step on.
             state[s] = 1;
@@ -110,15 +109,12 @@ k_springs(int64_t m, int64_t n, const int32_t *__restrict__ si, const int32_t *_
         } else {
             double cs;
             if constexpr (PREC == LSM_PREC_EXACT64) {
-                const double r = __dsqrt_rn(r2);
-                cs = dv(ml(t.k, sb(r, t.r0)), r);
                 if (SAMPLE) {
-                    const double e = sb(r, t.r0);
                     u = ml(ml(ml(0.5, t.k), e), e);
+                    w = ml(d[0], f[0]);
                 }
 #pragma unroll
-                for (int c = 0; c < DIM; c++) fs[c * m + s] = ml(cs, d[c]);
-                if (SAMPLE) w = ml(d[0], ml(cs, d[0]));
+                for (int c = 0; c < DIM; c++) fs[c * m + s] = f[c];
             } else if constexpr (PREC == LSM_PREC_FAST64) {
                 const double ir = rsqrt(r2);
                 cs = fma(-t.kr0, ir, t.k);  // k (r - r0) / r = k - k r0 / r
@@ -182,13 +178,13 @@ k_gather(int64_t n, int64_t m, const int64_t *__restrict__ row, const uint32_t *
         for (int64_t e = e0; e < e1; e++) {
             const uint32_t word = inc[e];
             const int64_t s = word >> 1;
-            if (word & 1u) {
+            // F - f is F + (-f): the sign goes onto the term (an integer
+            // operation), so that a warp whose lanes stand at upper and lower
+            // ends takes one FP64 addition and not one of each kind
+            const unsigned long long flip = (unsigned long long)(word & 1u) << 63;
 #pragma unroll
-                for (int c = 0; c < DIM; c++) F[c] = sb(F[c], fs[c * m + s]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < DIM; c++) F[c] = ad(F[c], fs[c * m + s]);
-            }
+            for (int c = 0; c < DIM; c++)
+                F[c] = ad(F[c], __longlong_as_double(__double_as_longlong(fs[c * m + s]) ^ (long long)flip));
         }
         const uint8_t fx = fixm[p];
         const double mp = mass[p];
@@ -199,7 +195,7 @@ k_gather(int64_t n, int64_t m, const int64_t *__restrict__ row, const uint32_t *
             if (SAMPLE && c == 0 && grip[p] == 2) react = sb(react, F[0]);
             if (fx & (1u << c)) continue;
             if constexpr (MODE == G_INIT) {
-                a[q] = dv(sb(F[c], ml(gamma, v[q])), mp);
+                a[q] = e64_div_mass(sb(F[c], ml(gamma, v[q])), mp);
             } else if constexpr (MODE == G_OBSERVE) {
                 const double vn = v[q];
                 if (SAMPLE) {
@@ -209,7 +205,7 @@ k_gather(int64_t n, int64_t m, const int64_t *__restrict__ row, const uint32_t *
                 }
             } else {
                 const double vh = v[q];
-                const double acc = dv(sb(F[c], ml(gamma, vh)), mp);
+                const double acc = e64_div_mass(sb(F[c], ml(gamma, vh)), mp);
                 const double vn = ad(vh, ml(hdt, acc));
                 if (SAMPLE) {
                     res = fmax(res, fmax(fabs(F[c]), fabs(vn)));

@@ -8,6 +8,7 @@
 #include <type_traits>
 
 #include "dfloat.cuh"
+#include "exact64.cuh"
 #include "lsm_internal.h"
 
 namespace lsm {
@@ -28,7 +29,6 @@ __host__ __device__ constexpr int tile_threads()
 __device__ __forceinline__ double ad(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ double sb(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double ml(double a, double b) { return __dmul_rn(a, b); }
-__device__ __forceinline__ double dv(double a, double b) { return __ddiv_rn(a, b); }
 
 template <int NWARP>
 __device__ __forceinline__ double bsum(double v, double *sh)
@@ -271,19 +271,17 @@ __device__ __forceinline__ void eval_spring(const TileArgs &A, int rp, int rq, i
         bool brk_now = false;
         if constexpr (PREC == LSM_PREC_EXACT64) {
             const SpringType t = stab[ti];
-            const double ddx = sb(sx[rq], sx[rp]), ddy = sb(sy[rq], sy[rp]);
-            const double r2 = ad(ml(ddx, ddx), ml(ddy, ddy));
-            if (MODE == T_STEP && r2 > t.rc2) {
+            const double d[2] = {sb(sx[rq], sx[rp]), sb(sy[rq], sy[rp])};
+            double r2, st, f[2];  // st = r - r0
+            e64_force<2>(d, t.k, t.r0, r2, st, f);
+            if (MODE == T_STEP && e64_gt(r2, t.rc2)) {
                 brk_now = true;
             } else {
-                const double r = __dsqrt_rn(r2);
-                const double c = dv(ml(t.k, sb(r, t.r0)), r);
-                fx = ml(c, ddx);
-                fy = ml(c, ddy);
+                fx = f[0];
+                fy = f[1];
                 if (SAMPLE && OWNER) {
-                    const double st = sb(r, t.r0);
                     u_acc += ml(ml(ml(0.5, t.k), st), st);
-                    w_acc += ml(ddx, ml(c, ddx));
+                    w_acc += ml(d[0], fx);
                 }
             }
         } else if constexpr (PREC == LSM_PREC_FAST64) {
@@ -622,7 +620,7 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
             const double vh = MODE == T_INIT ? A.v_obs[q] : A.vh_in[q];
             double vn, vh2;
             if constexpr (PREC == LSM_PREC_EXACT64) {
-                const double acc = dv(sb(F[c], ml(A.gamma, vh)), m);
+                const double acc = e64_div_mass(sb(F[c], ml(A.gamma, vh)), m);
                 vn = ad(vh, ml(A.hdt, acc));
                 vh2 = ad(vn, ml(A.hdt, acc));
             } else {
