@@ -117,14 +117,18 @@ cudaError_t tile_export(Ctx &c, bool steps)
 
 constexpr int TILE_X = 32;
 
-// Tile height: 8 rows of one warp each (6 CTAs per SM) for the double-float
+// Tile height: 8 rows of one warp each for the double-float and exact FP64
 // steps without a sample, 16 rows otherwise (measured fastest per mode on the
-// 2048 x 2048 composite). Only sample steps write per-tile partial sums, so
-// the partials always come from 16-row tiles (half as many block reductions
+// 2048 x 2048 composite). An exact 16-row tile takes 50 KB of shared memory, so
+// only 4 CTAs share an SM and the FP64 pipe idles in each one's load and gather
+// phases; 8-row tiles (27 KB, 5 CTAs by registers) take it from 62% to 70% busy
+// (2048^2 488 -> 481 us, 1000 x 700 93 -> 88 us) and give a small image twice the
+// CTAs (64^2: 19.1 -> 11.7 us). Only sample steps write per-tile partial sums,
+// so the partials always come from 16-row tiles (half as many block reductions
 // as 8-row tiles would need).
 constexpr int TILE_Y_SAMPLE = 16;
 template <int PREC, bool SAMPLE>
-constexpr int tile_y() { return PREC == LSM_PREC_DF && !SAMPLE ? 8 : TILE_Y_SAMPLE; }
+constexpr int tile_y() { return (PREC == LSM_PREC_DF || PREC == LSM_PREC_EXACT64) && !SAMPLE ? 8 : TILE_Y_SAMPLE; }
 
 static TileArgs tile_args(Ctx &c)
 {
