@@ -58,9 +58,9 @@ typedef enum {
  *      fused multiply-add, gather in canonical spring order: the same
  *      operations in the same order as the plain FP64 definition, so the
  *      state is bit-identical to a sequential FP64 evaluation.
- *  LSM_PREC_FAST64: double precision throughout, reassociated (fused
- *      multiply-add, 1/r from a reciprocal square root); results agree with
- *      the exact mode to a few ulps per step.
+ *  LSM_PREC_FAST64: double precision throughout, in whatever order and form
+ *      is fastest; results agree with the exact mode to a few ulps per step.
+ *      At present the exact kernels are, and this mode runs them.
  *  LSM_PREC_F32: spring vector formed exactly (positions in 64-bit fixed
  *      point), spring force evaluated and gathered in single precision,
  *      positions and velocities integrated in double.

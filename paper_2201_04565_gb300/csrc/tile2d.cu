@@ -19,10 +19,10 @@
 // flags are the low 4 bits of mask[p], written only by the tile owning p.
 //
 // Precision modes: EXACT64 performs the same correctly rounded operations in
-// the same order as the sequential FP64 definition (bit-identical state);
-// FAST64 uses fused multiply-add and a reciprocal square root; F32 and DF form
-// the spring vector exactly from 64-bit fixed-point positions and evaluate the
-// force in single precision or in double-float arithmetic, integrating in FP64.
+// the same order as the sequential FP64 definition (bit-identical state), and
+// FAST64 runs on it; F32 and DF form the spring vector exactly from 64-bit
+// fixed-point positions and evaluate the force in single precision or in
+// double-float arithmetic, integrating in FP64.
 #include "tile_body.cuh"
 
 #include <cmath>
@@ -200,11 +200,13 @@ static cudaError_t launch_tile(Ctx &c, TileArgs A)
 
 // constant strain-rate loading is a separate instance of the time step, so
 // that the ordinary step carries none of its code (registers)
+// FAST64 runs the exact kernel, which is the faster one since its root and
+// division left the FP64 pipe (1000 x 700: 88 us a step; fused multiply-adds
+// and rsqrt on that pipe took 113 us).
 template <int MODE, bool SAMPLE, bool RATE>
 static cudaError_t launch_tile_p(Ctx &c, TileArgs A)
 {
     switch (c.h.precision) {
-    case LSM_PREC_FAST64: return launch_tile<LSM_PREC_FAST64, MODE, SAMPLE, RATE>(c, A);
     case LSM_PREC_F32: return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE>(c, A);
     case LSM_PREC_DF: return launch_tile<LSM_PREC_DF, MODE, SAMPLE, RATE>(c, A);
     default: return launch_tile<LSM_PREC_EXACT64, MODE, SAMPLE, RATE>(c, A);

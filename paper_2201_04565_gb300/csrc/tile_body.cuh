@@ -131,7 +131,7 @@ struct TileArgs {
 
 // CTAs per SM the 8- and 16-row tile kernels are compiled for: 3 of 16
 // warps for the 16-row double-float time step, 6 of 8 warps for the other
-// double-float, FP32 and FAST64 steps, 5 for the exact FP64 step, 4 of 8
+// double-float and FP32 steps, 5 for the exact FP64 step, 4 of 8
 // warps for every sample step (the register budgets that leave, 42, 51 and 64
 // per thread, hold each kernel without spills, up to 12 bytes in the batched
 // FP32 step)
@@ -282,23 +282,6 @@ __device__ __forceinline__ void eval_spring(const TileArgs &A, int rp, int rq, i
                 if (SAMPLE && OWNER) {
                     u_acc += ml(ml(ml(0.5, t.k), st), st);
                     w_acc += ml(d[0], fx);
-                }
-            }
-        } else if constexpr (PREC == LSM_PREC_FAST64) {
-            const SpringType t = stab[ti];
-            const double ddx = sx[rq] - sx[rp], ddy = sy[rq] - sy[rp];
-            const double r2 = fma(ddx, ddx, ddy * ddy);
-            if (MODE == T_STEP && r2 > t.rc2) {
-                brk_now = true;
-            } else {
-                const double ir = rsqrt(r2);
-                const double c = fma(-t.kr0, ir, t.k);
-                fx = c * ddx;
-                fy = c * ddy;
-                if (SAMPLE && OWNER) {
-                    const double st = fma(r2, ir, -t.r0);
-                    u_acc += 0.5 * t.k * st * st;
-                    w_acc += ddx * fx;
                 }
             }
         } else {
@@ -572,13 +555,9 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
                 acc += sf[(c * 4 + 1) * NS + rp] - sf[(c * 4 + 2) * NS + s2];
                 acc += sf[(c * 4 + 2) * NS + rp] - sf[(c * 4 + 1) * NS + s1];
                 acc += sf[(c * 4 + 3) * NS + rp] - sf[(c * 4 + 0) * NS + s0];
-                if constexpr (PREC == LSM_PREC_F32) {
-                    F[c] = f2d_force(acc);
-                    Ff[c] = acc;
-                    Fd[c] = ff{acc, 0.0f};
-                } else {
-                    F[c] = acc;
-                }
+                F[c] = f2d_force(acc);
+                Ff[c] = acc;
+                Fd[c] = ff{acc, 0.0f};
             }
         }
         const bool grip = gx == 0 || gx == A.nx - 1;
@@ -587,9 +566,8 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
         const double m = smass[ph];
         const double xr[2] = {opx[k], opy[k]};
         if (SAMPLE && gx == A.nx - 1) {
-            if constexpr (PREC == LSM_PREC_EXACT64) react = sb(react, F[0]);
-            else if constexpr (FIX) reactf = ff_add_sloppy(reactf, ff_neg(Fd[0]));
-            else react -= F[0];
+            if constexpr (FIX) reactf = ff_add_sloppy(reactf, ff_neg(Fd[0]));
+            else react = sb(react, F[0]);
         }
 #pragma unroll
         for (int c = 0; c < 2; c++) {
