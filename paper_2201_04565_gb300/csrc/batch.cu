@@ -6,10 +6,13 @@
 // step is one launch of k_tile2d_batch over a global tile list; CTAs walk the
 // list with a grid stride, so the grid can be one CTA per tile or a
 // persistent grid. Every specimen has its own ping-pong parity, step counter
-// and "active" flag (relax stops stepping converged specimens); a tiny kernel
-// after each step flips the parity of the active ones. Samples are folded per
-// specimen from that specimen's contiguous range of per-tile partial sums, in
-// a fixed order.
+// and "active" flag (relax stops stepping converged specimens). Activity does
+// not change within a call's steps, so step t of a call takes its parity and
+// step index from the specimen's values at the start of the call and t, and
+// the reduction that ends the call advances both (a kernel that did so after
+// every step cost its launch each time: 13.2 -> 11.7 us a step on 12 specimens of
+// 128^2). Samples are folded per specimen from that specimen's contiguous
+// range of per-tile partial sums, in a fixed order.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(tile_threads<TY, PREC, SAMPLE>(), (tile_min_ct
 k_tile2d_batch(TileArgs base, const BatchTile *__restrict__ tiles, int64_t t0, int64_t t1,
                const SpecDesc *__restrict__ specs, double *X0, double *X1, double *V0, double *V1, double *VOBS,
                const uint8_t *PH, uint8_t *MASK, long long *BRK, unsigned long long *fb,
-               unsigned long long *nb)
+               unsigned long long *nb, int step)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     for (int64_t t = t0 + blockIdx.x; t < t1; t += gridDim.x) {
@@ -109,8 +112,9 @@ k_tile2d_batch(TileArgs base, const BatchTile *__restrict__ tiles, int64_t t0, i
         A.nx = sd.nx;
         A.ny = sd.ny;
         A.np = (int64_t)sd.nx * sd.ny;
-        double *xa = (sd.cur ? X1 : X0) + 2 * P, *xb = (sd.cur ? X0 : X1) + 2 * P;
-        double *va = (sd.cur ? V1 : V0) + 2 * P, *vb = (sd.cur ? V0 : V1) + 2 * P;
+        const bool odd = (sd.cur ^ step) & 1;  // parity at this step of the call
+        double *xa = (odd ? X1 : X0) + 2 * P, *xb = (odd ? X0 : X1) + 2 * P;
+        double *va = (odd ? V1 : V0) + 2 * P, *vb = (odd ? V0 : V1) + 2 * P;
         A.x_in = xa;
         A.vh_in = va;
         A.x_out = xb;
@@ -122,7 +126,7 @@ k_tile2d_batch(TileArgs base, const BatchTile *__restrict__ tiles, int64_t t0, i
         A.first_break = fb + bt.spec;
         A.nbroken = nb + bt.spec;
         A.d_step = &specs[bt.spec].steps;
-        A.t_off = 0;
+        A.t_off = step;
         tile_body<32, TY, PREC, MODE, SAMPLE>(A, bt.bx, bt.by, t, smem_raw);
         __syncthreads();
     }
@@ -139,7 +143,8 @@ template <int PREC, bool SAMPLE>
 __global__ void __launch_bounds__(32 * STRIP_WARPS, 5)
 k_strip2d_batch(TileArgs base, const BatchTile *__restrict__ strips, int64_t n, int R,
                 const SpecDesc *__restrict__ specs, double *X0, double *X1, double *V0, double *V1, double *VOBS,
-                const uint8_t *PH, uint8_t *MASK, long long *BRK, unsigned long long *fb, unsigned long long *nb)
+                const uint8_t *PH, uint8_t *MASK, long long *BRK, unsigned long long *fb, unsigned long long *nb,
+                int step)
 {
     __shared__ TypeDF sdf[128];
     __shared__ Coef4 scoef[8];
@@ -158,10 +163,11 @@ k_strip2d_batch(TileArgs base, const BatchTile *__restrict__ strips, int64_t n, 
         A.nx = sd.nx;
         A.ny = sd.ny;
         A.np = (int64_t)sd.nx * sd.ny;
-        A.x_in = (sd.cur ? X1 : X0) + 2 * P;
-        A.x_out = (sd.cur ? X0 : X1) + 2 * P;
-        A.vh_in = (sd.cur ? V1 : V0) + 2 * P;
-        A.vh_out = (sd.cur ? V0 : V1) + 2 * P;
+        const bool odd = (sd.cur ^ step) & 1;  // parity at this step of the call
+        A.x_in = (odd ? X1 : X0) + 2 * P;
+        A.x_out = (odd ? X0 : X1) + 2 * P;
+        A.vh_in = (odd ? V1 : V0) + 2 * P;
+        A.vh_out = (odd ? V0 : V1) + 2 * P;
         A.v_obs = VOBS + 2 * P;
         A.phase = PH + P;
         A.mask = MASK + P;
@@ -169,18 +175,8 @@ k_strip2d_batch(TileArgs base, const BatchTile *__restrict__ strips, int64_t n, 
         A.first_break = fb + st.spec;
         A.nbroken = nb + st.spec;
         A.d_step = &specs[st.spec].steps;
-        A.t_off = 0;
+        A.t_off = step;
         strip_run<PREC, false, SAMPLE, 0, T_STEP>(A, R, st.bx, st.by * R, q, sdf, scoef, smassf, soff);
-    }
-}
-
-// After a step: active specimens advance their parity and step count.
-__global__ void k_batch_flip(SpecDesc *specs, int S)
-{
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < S && specs[s].active) {
-        specs[s].cur ^= 1;
-        specs[s].steps += 1;
     }
 }
 
@@ -190,13 +186,14 @@ __global__ void k_batch_set_active(SpecDesc *specs, int S, int v)
     if (s < S) specs[s].active = v;
 }
 
-// One block per specimen: fold its tiles' partials in a fixed order into a
-// sample. relax: specimens whose residual is <= tol stop stepping; nactive
+// One block per specimen: advance its parity and step count by the call's
+// steps (active specimens) and fold its tiles' partials in a fixed order into
+// a sample. relax: specimens whose residual is <= tol stop stepping; nactive
 // counts the ones still active.
 __global__ void __launch_bounds__(256)
 k_batch_reduce(SpecDesc *specs, const double *__restrict__ ps, const double *__restrict__ pp, int64_t T,
                const unsigned long long *__restrict__ nb, DeviceSample *dst, int64_t cap,
-               const long long *d_nsamp, int record, int relax, double tol, int *nactive)
+               const long long *d_nsamp, int record, int relax, double tol, int *nactive, long long nsteps)
 {
     __shared__ double sh[8];
     const int s = blockIdx.x;
@@ -214,6 +211,10 @@ k_batch_reduce(SpecDesc *specs, const double *__restrict__ ps, const double *__r
     double r[6];
     for (int q = 0; q < 6; q++) r[q] = q == 5 ? bmax<8>(acc[q], sh) : bsum<8>(acc[q], sh);
     if (threadIdx.x == 0) {
+        if (sd.active) {
+            sd.cur ^= (int)(nsteps & 1);
+            sd.steps += nsteps;
+        }
         DeviceSample smp;
         smp.eps = sd.eps;
         smp.sigma_vir = (r[0] - r[2]) / sd.omega;
@@ -490,19 +491,19 @@ static bool batch_strips_fill(const BatchCtx &b, int R)
 }
 
 template <int PREC, bool SAMPLE>
-static cudaError_t launch_bs(BatchCtx &b)
+static cudaError_t launch_bs(BatchCtx &b, int64_t step)
 {
     if (b.NSTRIP <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)((b.NSTRIP + STRIP_WARPS - 1) / STRIP_WARPS);  // one warp per strip
     k_strip2d_batch<PREC, SAMPLE><<<grid, 32 * STRIP_WARPS, 0, b.stream>>>(batch_base_args(b), b.strips, b.NSTRIP, b.strip_r,
                                                                     b.specs, b.X[0], b.X[1], b.VH[0], b.VH[1], b.VOBS,
-                                                                    b.PH, b.MASK, b.BRK, b.fb, b.nb);
+                                                                    b.PH, b.MASK, b.BRK, b.fb, b.nb, (int)step);
     b.launches += 1;
     return cudaGetLastError();
 }
 
 template <int TY, int PREC, int MODE, bool SAMPLE>
-static cudaError_t launch_bt(BatchCtx &b, const BatchTile *tiles, int64_t t0, int64_t t1)
+static cudaError_t launch_bt(BatchCtx &b, const BatchTile *tiles, int64_t t0, int64_t t1, int64_t step)
 {
     auto kern = k_tile2d_batch<TY, PREC, MODE, SAMPLE>;
     const size_t smem = tile_smem_bytes<32, TY>(PREC);
@@ -516,26 +517,28 @@ static cudaError_t launch_bt(BatchCtx &b, const BatchTile *tiles, int64_t t0, in
     if (ntl <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)(b.grid > 0 && b.grid < ntl ? b.grid : ntl);
     kern<<<grid, tile_threads<TY, PREC, SAMPLE>(), smem, b.stream>>>(batch_base_args(b), tiles, t0, t1, b.specs, b.X[0], b.X[1],
-                                                 b.VH[0], b.VH[1], b.VOBS, b.PH, b.MASK, b.BRK, b.fb, b.nb);
+                                                 b.VH[0], b.VH[1], b.VOBS, b.PH, b.MASK, b.BRK, b.fb, b.nb,
+                                                 (int)step);
     b.launches += 1;
     return cudaGetLastError();
 }
 
 // Steps without a sample run on the tile list of the schedule's height;
-// sample steps on the 16-row list (t0, t1 index the list used).
+// sample steps on the 16-row list (t0, t1 index the list used; step: index of
+// the time step within the call).
 template <int MODE, bool SAMPLE>
-static cudaError_t launch_b(BatchCtx &b, int64_t t0, int64_t t1)
+static cudaError_t launch_b(BatchCtx &b, int64_t t0, int64_t t1, int64_t step = 0)
 {
 #define BT_PREC(TYV, TL)                                                                          \
     switch (b.prec) {                                                                             \
     case LSM_PREC_EXACT64:                                                                        \
-    case LSM_PREC_FAST64: return launch_bt<TYV, LSM_PREC_EXACT64, MODE, SAMPLE>(b, TL, t0, t1);   \
-    case LSM_PREC_F32: return launch_bt<TYV, LSM_PREC_F32, MODE, SAMPLE>(b, TL, t0, t1);          \
-    default: return launch_bt<TYV, LSM_PREC_DF, MODE, SAMPLE>(b, TL, t0, t1);                     \
+    case LSM_PREC_FAST64: return launch_bt<TYV, LSM_PREC_EXACT64, MODE, SAMPLE>(b, TL, t0, t1, step);   \
+    case LSM_PREC_F32: return launch_bt<TYV, LSM_PREC_F32, MODE, SAMPLE>(b, TL, t0, t1, step);          \
+    default: return launch_bt<TYV, LSM_PREC_DF, MODE, SAMPLE>(b, TL, t0, t1, step);                     \
     }
     if (MODE == T_STEP && b.strip_r > 0) {  // time steps on strips
-        if (b.prec == LSM_PREC_F32) return launch_bs<LSM_PREC_F32, SAMPLE>(b);
-        return launch_bs<LSM_PREC_DF, SAMPLE>(b);
+        if (b.prec == LSM_PREC_F32) return launch_bs<LSM_PREC_F32, SAMPLE>(b, step);
+        return launch_bs<LSM_PREC_DF, SAMPLE>(b, step);
     }
     if constexpr (SAMPLE) {
         BT_PREC(16, b.stiles)
@@ -550,16 +553,13 @@ static cudaError_t launch_b(BatchCtx &b, int64_t t0, int64_t t1)
 // nsteps steps (+ sample on the last) and the per-specimen reduction.
 static cudaError_t enqueue_batch_steps(BatchCtx &b, int64_t nsteps, int record, int relax, double tol)
 {
-    const unsigned sg = (unsigned)((b.S + 255) / 256);
     for (int64_t t = 0; t < nsteps; t++) {
-        cudaError_t e = t == nsteps - 1 ? launch_b<T_STEP, true>(b, 0, b.TS) : launch_b<T_STEP, false>(b, 0, b.T);
+        cudaError_t e = t == nsteps - 1 ? launch_b<T_STEP, true>(b, 0, b.TS, t) : launch_b<T_STEP, false>(b, 0, b.T, t);
         if (e != cudaSuccess) return e;
-        k_batch_flip<<<sg, 256, 0, b.stream>>>(b.specs, b.S);
-        b.launches += 1;
     }
     k_batch_reduce<<<b.S, 256, 0, b.stream>>>(b.specs, b.part_s, b.part_p, b.TS, b.nb,
                                                record ? b.samples : b.scratch, b.cap, b.d_nsamp, record, relax, tol,
-                                               b.nactive);
+                                               b.nactive, (long long)nsteps);
     b.launches += 1;
     if (record) {
         k_batch_count<<<1, 1, 0, b.stream>>>(b.d_nsamp);
