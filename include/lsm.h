@@ -105,7 +105,8 @@ enum { LSM_PREC_EXACT64 = 0, LSM_PREC_FAST64 = 1, LSM_PREC_F32 = 2, LSM_PREC_DF 
  *  precision    LSM_PREC_* (see above).
  *  path         0 = automatic: images with up to 8 phases run on the grid
  *               of their pixels or sites. Square lattice: the fused tile
- *               kernel in every mode; in the F32 and DF modes, when the
+ *               kernel in every mode (images too small to fill the device:
+ *               up to three time steps per launch); in the F32 and DF modes, when the
  *               image is large enough for its strips to fill the device,
  *               the time steps run on the register-resident strip kernel
  *               instead (the same positions, velocities and breaks; sample
@@ -113,7 +114,8 @@ enum { LSM_PREC_EXACT64 = 0, LSM_PREC_FAST64 = 1, LSM_PREC_F32 = 2, LSM_PREC_DF 
  *               strip kernel. 3D (F32, DF): the voxel tile kernel.
  *               Everything else: the general spring-list kernels.
  *               1 = always the general spring-list kernels;
- *               2 = as 0, but every square-lattice 2D step on the tile kernel;
+ *               2 = as 0, but every square-lattice 2D step on the tile
+ *               kernel, one step per launch;
  *               3 = as 0, but the 2D F32 / DF steps on the strip kernel
  *               whatever the image size.
  *  stream       cudaStream_t to order work on (NULL = the library creates one).

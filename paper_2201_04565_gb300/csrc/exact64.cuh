@@ -292,39 +292,70 @@ __device__ __forceinline__ double e64_div_mass(double x, double m)
     return e64_bits(m) == 0x3FF0000000000000ull ? x : e64_div_fp64(x, m);
 }
 
-// One spring from its vector d: r2 = |d|^2 (components in order), the stretch
-// e = sqrt(r2) - r0, and the force f = ((k e) / sqrt(r2)) d on the lower end,
-// every operation rounded as IEEE double. Left on the FP64 pipe: the sum of
+// NS springs from their vectors d: r2 = |d|^2 (components in order), the
+// stretch e = sqrt(r2) - r0, and the force f = ((k e) / sqrt(r2)) d on the lower
+// end, every operation rounded as IEEE double. Left on the FP64 pipe: the sum of
 // the squares and the subtraction of r0. Where an operand is outside the
-// ranges above, all of it is done again there.
+// ranges above, all of that spring is done again there. The springs go through
+// each stage together and without branches, so that their dependent chains
+// (some 500 instructions each) overlap where few warps run.
+template <int DIM, int NS>
+__device__ __forceinline__ void e64_force_n(const double (&d)[NS][DIM], const double (&k)[NS], const double (&r0)[NS],
+                                            double (&r2)[NS], double (&e)[NS], double (&f)[NS][DIM])
+{
+    bool ok[NS];
+    Root64 r[NS];
+#pragma unroll
+    for (int s = 0; s < NS; s++) {
+        ok[s] = true;
+        r2[s] = e64_sqr(e64_bits(d[s][0]), ok[s]);
+#pragma unroll
+        for (int c = 1; c < DIM; c++) r2[s] = __dadd_rn(r2[s], e64_sqr(e64_bits(d[s][c]), ok[s]));
+    }
+#pragma unroll
+    for (int s = 0; s < NS; s++) {
+        const uint64_t x = e64_bits(r2[s]);
+        ok[s] = ok[s] && (unsigned)((int)(x >> 52) - 1) < 2046u;  // positive and normal
+        float y;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(e64_sqrt_arg(x)));
+        r[s] = e64_sqrt(x, y);
+        e[s] = __dsub_rn(e64_root(r[s]), r0[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < NS; s++) {
+        uint64_t ke = e64_bits(e[s]);
+        if (NS > 1 || e64_bits(k[s]) != 0x3FF0000000000000ull) ke = e64_bits(e64_mul(e64_bits(k[s]), ke, ok[s]));
+        const bool zero = e64_zero(ke);  // 0 / r = 0
+        ok[s] = ok[s] && (zero || e64_div_ok(ke, r[s]));
+        const uint64_t c = zero ? ke : e64_bits(e64_div(ke, r[s]));
+#pragma unroll
+        for (int q = 0; q < DIM; q++) f[s][q] = e64_mul(c, e64_bits(d[s][q]), ok[s]);
+    }
+#pragma unroll
+    for (int s = 0; s < NS; s++)
+        if (!ok[s]) {
+            const Spring64 h = e64_force_fp64(d[s][0], d[s][1], DIM == 3 ? d[s][DIM - 1] : 0.0, k[s], r0[s]);
+            r2[s] = h.r2;
+            e[s] = h.e;
+#pragma unroll
+            for (int q = 0; q < DIM; q++) f[s][q] = h.f[q];
+        }
+}
+
+// One spring.
 template <int DIM>
 __device__ __forceinline__ void e64_force(const double (&d)[DIM], double k, double r0, double &r2, double &e,
                                           double (&f)[DIM])
 {
-    bool ok = true;
-    r2 = e64_sqr(e64_bits(d[0]), ok);
+    double dn[1][DIM], fn[1][DIM], r2n[1], en[1];
+    const double kn[1] = {k}, r0n[1] = {r0};
 #pragma unroll
-    for (int c = 1; c < DIM; c++) r2 = __dadd_rn(r2, e64_sqr(e64_bits(d[c]), ok));
-    const uint64_t x = e64_bits(r2);
-    ok = ok && (unsigned)((int)(x >> 52) - 1) < 2046u;  // positive and normal
-    float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(e64_sqrt_arg(x)));
-    const Root64 r = e64_sqrt(x, y);
-    e = __dsub_rn(e64_root(r), r0);
-    uint64_t ke = e64_bits(e);
-    if (e64_bits(k) != 0x3FF0000000000000ull) ke = e64_bits(e64_mul(e64_bits(k), ke, ok));
-    const bool zero = e64_zero(ke);  // 0 / r = 0
-    ok = ok && (zero || e64_div_ok(ke, r));
-    const uint64_t c = zero ? ke : e64_bits(e64_div(ke, r));
+    for (int q = 0; q < DIM; q++) dn[0][q] = d[q];
+    e64_force_n<DIM, 1>(dn, kn, r0n, r2n, en, fn);
+    r2 = r2n[0];
+    e = en[0];
 #pragma unroll
-    for (int q = 0; q < DIM; q++) f[q] = e64_mul(c, e64_bits(d[q]), ok);
-    if (!ok) {
-        const Spring64 s = e64_force_fp64(d[0], d[1], DIM == 3 ? d[DIM - 1] : 0.0, k, r0);
-        r2 = s.r2;
-        e = s.e;
-#pragma unroll
-        for (int q = 0; q < DIM; q++) f[q] = s.f[q];
-    }
+    for (int q = 0; q < DIM; q++) f[q] = fn[0][q];
 }
 #endif
 

@@ -507,6 +507,8 @@ static cudaError_t upload_tile(Ctx &c)
             c.nstrips = 0;
         }
     }
+    // path 2 keeps the one-step tile kernel
+    if (!c.strip && !c.tri && c.path_req != 2) c.multi = multi_shape(h.precision, h.nx, h.ny);
     if (c.tri) c.ntiles = c.nstrips;  // the packing's samples all come from the strip kernel
     std::vector<double> X(2 * np);
     for (int64_t g = 0; g < np; g++) {
@@ -567,8 +569,8 @@ static cudaError_t upload_tile(Ctx &c)
     LSM_TRY(dalloc(&c.tinvm, 4 * h.nphase));
     LSM_TRY(dalloc(&c.tdf, tdf.size()));
     LSM_TRY(dalloc(&c.tsbase, np));
-    {  // partial sums: per tile (tile kernel samples) or per strip (strip samples)
-        const int64_t np_ = std::max<int64_t>(c.ntiles, c.nstrips);
+    {  // partial sums: per tile (tile and multi-step kernel samples) or per strip (strip samples)
+        const int64_t np_ = std::max(std::max<int64_t>(c.ntiles, c.nstrips), c.multi.tiles);
         LSM_TRY(dalloc(&c.part_s, 2 * np_));
         LSM_TRY(dalloc(&c.part_p, 4 * np_));
     }
@@ -716,13 +718,12 @@ static void gather(Ctx &c)
         c.h.damping, c.part_p, c.nblk_p, c.d_status, c.d_step);
 }
 
-// Fold the partial sums of the last sample kernel into one sample. strips:
-// they came from a strip-kernel step (one partial per strip), not from the
-// tile kernel (one per tile) or the spring-list kernels (one per block).
-static void reduce(Ctx &c, DeviceSample *dst, long long *counter, long long add_steps, bool strips = false)
+// Fold the partial sums of the last sample kernel into one sample; parts: how
+// many there are on the tile paths (the spring lists: one per block).
+static void reduce(Ctx &c, DeviceSample *dst, long long *counter, long long add_steps, int64_t parts = 0)
 {
-    const int64_t nbs = strips ? c.nstrips : c.tile ? c.ntiles : (c.m ? c.nblk_s : 1);
-    const int64_t nbp = strips ? c.nstrips : c.tile ? c.ntiles : c.nblk_p;
+    const int64_t nbs = c.tile ? parts : (c.m ? c.nblk_s : 1);
+    const int64_t nbp = c.tile ? parts : c.nblk_p;
     k_reduce<<<1, RED_THREADS, 0, c.stream>>>(c.part_s, nbs, c.part_p, nbp, c.d_eps, c.d_nbroken,
                                               c.d_step, add_steps, c.h.omega, c.h.grip_area, dst,
                                               counter, c.sample_cap, c.rate_on, c.rate_eps0, c.rate_step0,
@@ -755,15 +756,17 @@ static void enqueue_steps(Ctx &c, int64_t nsteps, bool record)
         reduce(c, c.scratch_sample, nullptr, 0);
 }
 
-static cudaError_t enqueue_tile_steps(Ctx &c, int64_t nsteps, bool record)
+static cudaError_t enqueue_tile_steps(Ctx &c, int64_t nsteps, bool record, int &end_buf)
 {
-    cudaError_t e = c.dim == 3 ? tile3_enqueue_steps(c, nsteps, c.tcur) : tile_enqueue_steps(c, nsteps, c.tcur);
+    cudaError_t e = c.dim == 3 ? tile3_enqueue_steps(c, nsteps, c.tcur, end_buf)
+                               : tile_enqueue_steps(c, nsteps, c.tcur, end_buf);
     if (e != cudaSuccess) return e;
-    const bool strips = c.dim == 2 && c.strip;  // the sample step ran on the strip kernel
+    // partial sums of the sample: per tile of the kernel that it ran on, or per strip
+    const int64_t parts = c.dim == 3 ? c.ntiles : c.strip ? c.nstrips : c.multi.shape ? c.multi.tiles : c.ntiles;
     if (record)
-        reduce(c, c.samples, c.d_nsamples, nsteps, strips);
+        reduce(c, c.samples, c.d_nsamples, nsteps, parts);
     else
-        reduce(c, c.scratch_sample, nullptr, nsteps, strips);
+        reduce(c, c.scratch_sample, nullptr, nsteps, parts);
     return cudaGetLastError();
 }
 
@@ -776,7 +779,7 @@ cudaError_t launch_steps(Ctx &c, int64_t nsteps, bool record)
         LSM_TRY(cudaStreamBeginCapture(c.stream, cudaStreamCaptureModeThreadLocal));
         cudaError_t ee = cudaSuccess;
         if (c.tile)
-            ee = enqueue_tile_steps(c, nsteps, record);
+            ee = enqueue_tile_steps(c, nsteps, record, c.graph_buf[key]);
         else if (c.dim == 3)
             enqueue_steps<3>(c, nsteps, record);
         else
@@ -798,7 +801,7 @@ cudaError_t launch_steps(Ctx &c, int64_t nsteps, bool record)
     }
     LSM_TRY(cudaGraphLaunch(it->second, c.stream));
     c.launches += c.graph_nodes[key];
-    if (c.tile) c.tcur ^= (int)(nsteps & 1);
+    if (c.tile) c.tcur = c.graph_buf[key];
     return cudaGetLastError();
 }
 
@@ -824,7 +827,7 @@ cudaError_t launch_observe(Ctx &c, DeviceSample *dst)
     if (c.tile) {
         cudaError_t e = c.dim == 3 ? tile3_observe(c) : tile_observe(c);
         if (e != cudaSuccess) return e;
-        reduce(c, dst, nullptr, 0);
+        reduce(c, dst, nullptr, 0, c.ntiles);
         return cudaGetLastError();
     }
     if (c.dim == 3) {

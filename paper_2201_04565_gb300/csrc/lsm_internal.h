@@ -120,6 +120,17 @@ struct HostNet {
     std::vector<double> offv;      // lattice vectors (x, y, z) by offset index (image builds)
 };
 
+// The multi-step tile kernel (tile_multi.cu): tile shape, the halo that bounds
+// the steps per launch, and the tiles of the image.
+enum { MULTI_NONE = 0, MULTI_16x4, MULTI_32x8, MULTI_E16x4, MULTI_E32x4 };
+struct MultiPlan {
+    int shape = MULTI_NONE;
+    int halo = 0;
+    int64_t tiles = 0;
+};
+MultiPlan multi_shape(int prec, int nx, int ny);
+
+
 struct Ctx {
     HostNet h;  // host copy of topology (kept for queries and rebuilds)
     int dim = 2;
@@ -224,6 +235,8 @@ struct Ctx {
     int64_t steps = 0; // host mirror of the step counter
     int64_t launches = 0;  // kernels launched (graph nodes included)
     std::map<int64_t, int64_t> graph_nodes;  // kernels per cached graph
+    MultiPlan multi;                         // multi-step tile kernel (small 2D images)
+    std::map<int64_t, int> graph_buf;        // state buffer that a cached graph ends in
     std::map<int64_t, cudaGraphExec_t> graphs;
 };
 
@@ -279,7 +292,7 @@ void fields_free(Ctx &c);
 
 // tile3d.cu: 3D voxel lattices in the fixed-point modes (state on the voxel grid)
 cudaError_t tile3_upload(Ctx &c);
-cudaError_t tile3_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf);
+cudaError_t tile3_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf, int &end_buf);
 cudaError_t tile3_init_accel(Ctx &c);
 cudaError_t tile3_observe(Ctx &c);
 cudaError_t tile3_export(Ctx &c, bool steps);
@@ -291,7 +304,7 @@ bool strip_supported(const Ctx &c);
 cudaError_t strip_geometry(Ctx &c, bool *fills);  // strip_R, strip_nsx, nstrips for this device
 
 // tile2d.cu
-cudaError_t tile_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf);
+cudaError_t tile_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf, int &end_buf);
 cudaError_t tile_init_accel(Ctx &c);
 cudaError_t tile_observe(Ctx &c);
 cudaError_t tile_apply_strain(Ctx &c, double eps_old, double eps_new);

@@ -220,9 +220,27 @@ static cudaError_t launch_tile_prec(Ctx &c, TileArgs A)
     return launch_tile_p<MODE, SAMPLE, false>(c, A);
 }
 
-cudaError_t tile_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf)
+cudaError_t tile_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf, int &end_buf)
 {
     int cur = start_buf;
+    if (c.multi.shape != MULTI_NONE) {  // up to multi.halo steps a launch, as evenly as they divide
+        for (int64_t t = 0; t < nsteps;) {
+            const int64_t left = nsteps - t, launches = (left + c.multi.halo - 1) / c.multi.halo;
+            const int ns = (int)((left + launches - 1) / launches);
+            TileArgs A = tile_args(c);
+            A.t_off = t;
+            A.x_in = c.tx[cur];
+            A.vh_in = c.tvh[cur];
+            A.x_out = c.tx[cur ^ 1];
+            A.vh_out = c.tvh[cur ^ 1];
+            const cudaError_t e = launch_multi(c, A, ns, t + ns == nsteps);
+            if (e != cudaSuccess) return e;
+            t += ns;
+            cur ^= 1;
+        }
+        end_buf = cur;
+        return cudaGetLastError();
+    }
     for (int64_t t = 0; t < nsteps; t++) {
         TileArgs A = tile_args(c);
         A.t_off = t;
@@ -237,6 +255,7 @@ cudaError_t tile_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf)
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
+    end_buf = cur;
     return cudaGetLastError();
 }
 

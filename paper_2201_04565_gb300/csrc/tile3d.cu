@@ -583,7 +583,7 @@ cudaError_t tile3_upload(Ctx &c)
     return cudaSuccess;
 }
 
-cudaError_t tile3_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf)
+cudaError_t tile3_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf, int &end_buf)
 {
     int cur = start_buf;
     for (int64_t t = 0; t < nsteps; t++) {
@@ -597,6 +597,7 @@ cudaError_t tile3_enqueue_steps(Ctx &c, int64_t nsteps, int start_buf)
         if (e != cudaSuccess) return e;
         cur ^= 1;
     }
+    end_buf = cur;
     return cudaGetLastError();
 }
 

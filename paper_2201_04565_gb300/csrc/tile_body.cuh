@@ -678,6 +678,10 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
 cudaError_t launch_strip(Ctx &c, const TileArgs &A, bool sample);
 cudaError_t launch_strip_mode(Ctx &c, const TileArgs &A, int mode);  // T_INIT / T_OBSERVE, triangular packing
 
+// tile_multi.cu: up to c.multi.halo time steps in one launch (small square-
+// lattice images); the same states as the tile kernel.
+cudaError_t launch_multi(Ctx &c, const TileArgs &A, int ns, bool sample);
+
 // Pixel-grid broken flags -> canonical spring order (defined in tile2d.cu).
 __global__ void k_tile_export(int nx, int ny, int64_t np, const uint8_t *__restrict__ phase,
                               const uint8_t *__restrict__ mask, const long long *__restrict__ brk,
