@@ -120,6 +120,12 @@ struct HostNet {
     std::vector<double> offv;      // lattice vectors (x, y, z) by offset index (image builds)
 };
 
+// Sums of a sample on their way into it (k_reduce).
+struct ReduceScratch {
+    double tot[6];
+    unsigned done;
+};
+
 // The multi-step tile kernel (tile_multi.cu): tile shape, the halo that bounds
 // the steps per launch, and the tiles of the image.
 enum { MULTI_NONE = 0, MULTI_16x4, MULTI_32x8, MULTI_E16x4, MULTI_E32x4 };
@@ -168,6 +174,7 @@ struct Ctx {
     int64_t sample_cap = 0;
     int64_t nsamples = 0;  // host mirror
     DeviceSample *scratch_sample = nullptr;
+    ReduceScratch *red = nullptr;
 
     // 2D tile path (image lattices): state on the pixel grid, ping-pong
     bool tile = false;
