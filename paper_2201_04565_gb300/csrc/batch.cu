@@ -86,6 +86,7 @@ struct BatchCtx {
     int64_t export_cap = 0;
     int64_t cap = 0, nsamples = 0;
     int fix_S = 40;
+    DfSplit df;
     long long a_fix = 0;
     int64_t spring_updates = 0, launches = 0;
     std::map<int64_t, cudaGraphExec_t> graphs;
@@ -469,6 +470,8 @@ static TileArgs batch_base_args(BatchCtx &b)
     A.p24 = ldexpf(1.0f, 24 - b.fix_S);
     A.p0 = ldexpf(1.0f, -b.fix_S);
     A.df_bias = (unsigned)(896 + 24 - b.fix_S) << 20;
+    A.df_M = (float)std::ldexp(1.5 * b.df.unit, 23 + b.fix_S - 24);
+    A.df_cmax = (float)b.df.cmax;
     A.status = b.status;
     A.part_s = b.part_s;
     A.part_p = b.part_p;
@@ -628,6 +631,7 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     b.fix_S = std::min(61 - (int)std::ceil(std::log2(extent)), 47 - (int)std::ceil(std::log2(b.a * std::sqrt(2.0))));
     b.fix_S = std::min(b.fix_S, 47 - (int)std::floor(std::log2(max_critical_length(h0.types))));
     b.a_fix = std::llround(std::ldexp(b.a, b.fix_S));
+    b.df = df_split(h0.types, 8);
     for (int q = 0; q < 2; q++) {
         BT_TRY(balloc(&b.X[q], 2 * NP));
         BT_TRY(balloc(&b.VH[q], 2 * NP));
@@ -722,11 +726,9 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     // default schedule: largest specimens first, plain steps on 16-row
     // strips in the fixed-point modes when the strips fill the device (what
     // the autotuner picks on the benchmark's batches; a warp sweeping a strip
-    // is latency-bound when few run), 16-row tiles otherwise; the exact FP64
-    // step on 8-row tiles (20 specimens of sides 32 to 512: 296 -> 283 us a
-    // step, 12 of 128: 37.4 -> 35.4 us; more CTAs per SM, as in tile2d.cu)
-    const int tiles_y = b.prec == LSM_PREC_EXACT64 || b.prec == LSM_PREC_FAST64 ? 8 : 16;
-    BT_TRY(build_tiles(b, batch_strips_ok(b) && batch_strips_fill(b, 16) ? -16 : tiles_y, 1));
+    // is latency-bound when few run), 8-row tiles otherwise (12 specimens of
+    // 128^2, a step: exact 37.4 -> 35.4 us against 16 rows, df64 11.3 -> 10.7)
+    BT_TRY(build_tiles(b, batch_strips_ok(b) && batch_strips_fill(b, 16) ? -16 : 8, 1));
     // initial acceleration of every specimen (vh = v + dt/2 a(0))
     {
         cudaError_t ei = launch_b<T_INIT, false>(b, 0, b.T);

@@ -67,6 +67,29 @@ inline double max_critical_length(const std::vector<SpringType> &types)
     return r;
 }
 
+// The DF force split (tile_body.cuh): forces are held as a multiple of a unit u
+// plus a remainder below u / 2, so that the multiples of a particle's forces
+// (`terms` at most) add without rounding while each is at most 2^24 u / terms. u is
+// the power of two that takes 1.5 times the largest tensile force of any type
+// (k (rc - r0), or 1/32 of k r0) into that range; a spring with |k (1 - r0/r)| up to
+// cmax stays in it (0 if no such limit exists: an unbreakable type).
+struct DfSplit {
+    double unit = 0x1p-21, cmax = 0.0;
+};
+inline DfSplit df_split(const std::vector<SpringType> &types, int terms)
+{
+    double f = 0.0, rc = 1.0;
+    for (const SpringType &t : types) {
+        const double r = std::sqrt(t.rc2);
+        rc = std::fmax(rc, r);
+        f = std::fmax(f, t.k * std::fmax(std::isfinite(r) ? r - t.r0 : 0.0, 0.03125 * t.r0));
+    }
+    DfSplit s;
+    s.unit = std::exp2(std::ceil(std::log2(f > 0.0 ? 1.5 * f * terms : 1.0)) - 24.0);
+    s.cmax = std::isfinite(rc) ? s.unit * 0x1p24 / terms / rc : 0.0;
+    return s;
+}
+
 // A double-float: the unevaluated sum hi + lo of two floats.
 struct ff {
     float hi, lo;
@@ -242,6 +265,7 @@ struct Ctx {
     int64_t steps = 0; // host mirror of the step counter
     int64_t launches = 0;  // kernels launched (graph nodes included)
     std::map<int64_t, int64_t> graph_nodes;  // kernels per cached graph
+    DfSplit df;                              // DF force split
     MultiPlan multi;                         // multi-step tile kernel (small 2D images)
     std::map<int64_t, int> graph_buf;        // state buffer that a cached graph ends in
     std::map<int64_t, cudaGraphExec_t> graphs;

@@ -33,6 +33,7 @@
 // to the next (the batch's sample steps stay on its tile list).
 #pragma once
 
+#include "df_pair.cuh"
 #include "tile_body.cuh"
 
 namespace lsm {
@@ -166,7 +167,7 @@ enum { S_NONE = 0, S_BREAK = 1, S_FORCE = 2 };
 template <int PREC, bool SAMPLE, bool TEST, int LAT, typename FT>
 __device__ __forceinline__ int strip_spring(const TileArgs &A, const PixFix &p, const PixFix &q, int slot,
                                             const TypeDF *sdf, const ff (*soff)[3], FT &fx, FT &fy, FT &dx,
-                                            FT &st, TypeDF &t)
+                                            FT &st, TypeDF &t, bool &big)
 {
     fx = FT{};
     fy = FT{};
@@ -176,7 +177,7 @@ __device__ __forceinline__ int strip_spring(const TileArgs &A, const PixFix &p, 
     t = sdf[(((int)(pp - 1) * A.nphase) + (int)(pq - 1)) * 2 + shell];
     bool b;
     if constexpr (PREC == LSM_PREC_DF) {
-        b = spring_df<TEST, SAMPLE>(q.xf - p.xf, q.yf - p.yf, t, A, fx, fy, dx, st);
+        b = spring_df<TEST, SAMPLE>(q.xf - p.xf, q.yf - p.yf, t, A, fx, fy, dx, st, big);
     } else if constexpr (LAT == 0) {
         b = spring_f32<TEST, SAMPLE>(q.xf - p.xf, q.yf - p.yf, slot, t, soff, A, fx, fy, dx, st);
     } else {
@@ -186,6 +187,49 @@ __device__ __forceinline__ int strip_spring(const TileArgs &A, const PixFix &p, 
                                        soff[slot][2].hi, t, A, fx, fy, dx, st);
     }
     return b ? S_BREAK : S_FORCE;
+}
+
+// Two forward springs of p (slots sa, sb; type shells sha, shb) at a time, DF time
+// steps: as strip_spring.
+__device__ __forceinline__ void strip_pair(const TileArgs &A, const PixFix &p, const PixFix &qa, int sa, int sha,
+                                           const PixFix &qb, int sb, int shb, const TypeDF *sdf, ff &fax, ff &fay,
+                                           ff &fbx, ff &fby, int &ra, int &rb, bool &big)
+{
+    const unsigned pp = p.pm & 0xffu, pa = qa.pm & 0xffu, pb = qb.pm & 0xffu;
+    const bool live[2] = {pp && pa && !((p.pm >> (8 + sa)) & 1u), pp && pb && !((p.pm >> (8 + sb)) & 1u)};
+    const int row = (int)(pp - 1) * A.nphase - 1;
+    const int ia = live[0] ? (row + (int)pa) * 2 + sha : 0, ib = live[1] ? (row + (int)pb) * 2 + shb : 0;
+    const long long d[2][2] = {{qa.xf - p.xf, qb.xf - p.xf}, {qa.yf - p.yf, qb.yf - p.yf}};
+    ff f[2][2];
+    bool brk[2];
+    spring_df_pair<2>(d, sdf[ia], sdf[ib], live, A.df_M, A.df_cmax, f, brk, big);
+    fax = f[0][0];
+    fbx = f[0][1];
+    fay = f[1][0];
+    fby = f[1][1];
+    ra = brk[0] ? S_BREAK : S_FORCE;
+    rb = brk[1] ? S_BREAK : S_FORCE;
+}
+
+// A particle's forces in the canonical order: square lattice incoming slots 3, 2,
+// 1, 0, packing 2, 1, 0, then its own.
+template <typename SUM, int LAT>
+__device__ __forceinline__ DfSum strip_sum(ff i3, ff i2, ff i1, ff i0, ff f0, ff f1, ff f2, ff f3)
+{
+    SUM s;
+    if constexpr (LAT == 0) {
+        s.first_neg(i3);
+        s.sub(i2);
+    } else {
+        s.first_neg(i2);
+    }
+    s.sub(i1);
+    s.sub(i0);
+    s.add(f0);
+    s.add(f1);
+    s.add(f2);
+    if constexpr (LAT == 0) s.add(f3);
+    return s;
 }
 
 // The sample sums of one intact spring: the potential energy and the
@@ -200,7 +244,7 @@ template <>
 __device__ __forceinline__ void spring_sample<ff>(ff &u, ff &w, const TypeDF &t, ff dx, ff fx, ff st)
 {
     u = ff_add_sloppy(u, ff_mul(t.k, ff_sqr(st)));
-    w = ff_add_sloppy(w, ff_mul(dx, fx));
+    w = ff_add_sloppy(w, ff_mul(dx, df_pair(fx)));
 }
 template <>
 __device__ __forceinline__ void spring_sample<float>(ff &u, ff &w, const TypeDF &t, float dx, float fx, float st)
@@ -300,6 +344,7 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
     raw = strip_fetch<VOBS>(A, gx, y0);
     double vcx = 0.0, vcy = 0.0;
     FT p1x{}, p1y{}, p2x{}, p2y{}, p3x{}, p3y{};  // previous row's forces (slots 1..3)
+    bool big_above = false;  // row y - 1 had a force beyond the split's exact range
     // square lattice: the slot-0 target (gx + 1, y) is the previous row's
     // slot-3 target (gx + 1, (y - 1) + 1), kept from its shuffle (not in the
     // sample step, whose sums need the registers)
@@ -341,13 +386,40 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
             if (lane == 31 && par) q3.pm = 0u;
         }
         const bool sum_springs = SAMPLE && own && owner;
-        FT f0x, f0y, dx, st;
-        TypeDF t;
-        const int s0 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q0, 0, sdf, soff, f0x, f0y, dx, st, t);
-        if (sum_springs && s0 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f0x, st);
+        FT f0x, f0y, f1x, f1y, f2x, f2y, f3x{}, f3y{};
+        int s0, s1, s2, s3 = S_NONE;
+        bool big = false;  // DF: a force beyond the split's exact range
+        if constexpr (PREC == LSM_PREC_DF && !SAMPLE && TEST) {
+            // two springs at a time on packed instructions (the same bits)
+            if constexpr (LAT == 0) {
+                strip_pair(A, P, q0, 0, 0, N, 2, 0, sdf, f0x, f0y, f2x, f2y, s0, s2, big);
+                strip_pair(A, P, q1, 1, 1, q3, 3, 1, sdf, f1x, f1y, f3x, f3y, s1, s3, big);
+            } else {
+                FT dx, st;
+                TypeDF t;
+                s0 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q0, 0, sdf, soff, f0x, f0y, dx, st, t, big);
+                strip_pair(A, P, q1, 1, 1, q3, 2, 1, sdf, f1x, f1y, f2x, f2y, s1, s2, big);
+            }
+        } else {
+            FT dx, st;
+            TypeDF t;
+            s0 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q0, 0, sdf, soff, f0x, f0y, dx, st, t, big);
+            if (sum_springs && s0 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f0x, st);
+            s1 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q1, 1, sdf, soff, f1x, f1y, dx, st, t, big);
+            if (sum_springs && s1 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f1x, st);
+            if constexpr (LAT == 0) {
+                s2 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, N, 2, sdf, soff, f2x, f2y, dx, st, t, big);
+                if (sum_springs && s2 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f2x, st);
+                s3 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q3, 3, sdf, soff, f3x, f3y, dx, st, t, big);
+                if (sum_springs && s3 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f3x, st);
+            } else {
+                s2 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q3, 2, sdf, soff, f2x, f2y, dx, st, t, big);
+                if (sum_springs && s2 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f2x, st);
+            }
+        }
+        // incoming springs: slot 0 of this row, the others of row y - 1
         const FT i0x = shfl_ft(f0x, lane - 1), i0y = shfl_ft(f0y, lane - 1);
-        // incoming springs of row y - 1
-        FT i3x, i3y, i1x, i1y, i2x, i2y;
+        FT i3x{}, i3y{}, i1x, i1y, i2x, i2y;
         if constexpr (LAT == 0) {
             i3x = shfl_ft(p3x, lane - 1);
             i3y = shfl_ft(p3y, lane - 1);
@@ -362,48 +434,11 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
             i1x = shfl_ft(p1x, lane + 1 - pp);
             i1y = shfl_ft(p1y, lane + 1 - pp);
         }
-
-        DfSum ax, ay;
-        float sx_ = 0.0f, sy_ = 0.0f;
+        bool careful = false;  // warp-uniform
         if constexpr (PREC == LSM_PREC_DF) {
-            if constexpr (LAT == 0) {  // canonical: slot 3, 2, 1 of row y - 1, slot 0 of row y
-                ax.first_neg(i3x);
-                ax.sub(i2x);
-                ay.first_neg(i3y);
-                ay.sub(i2y);
-            } else {  // canonical: slot 2, slot 1 of row y - 1, slot 0 of row y
-                ax.first_neg(i2x);
-                ay.first_neg(i2y);
-            }
-            ax.sub(i1x);
-            ax.sub(i0x);
-            ax.add(f0x);
-            ay.sub(i1y);
-            ay.sub(i0y);
-            ay.add(f0y);
-        } else {
-            if constexpr (LAT == 0) {
-                sx_ = f0x - i3x;
-                sy_ = f0y - i3y;
-            } else {
-                sx_ = f0x - i2x;
-                sy_ = f0y - i2y;
-            }
-        }
-        FT f1x, f1y, f2x, f2y, f3x{}, f3y{};
-        int s1, s2, s3 = S_NONE;
-        if constexpr (LAT == 0) {
-            s1 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q1, 1, sdf, soff, f1x, f1y, dx, st, t);
-            if (sum_springs && s1 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f1x, st);
-            s2 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, N, 2, sdf, soff, f2x, f2y, dx, st, t);
-            if (sum_springs && s2 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f2x, st);
-            s3 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q3, 3, sdf, soff, f3x, f3y, dx, st, t);
-            if (sum_springs && s3 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f3x, st);
-        } else {
-            s1 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q1, 1, sdf, soff, f1x, f1y, dx, st, t);
-            if (sum_springs && s1 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f1x, st);
-            s2 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q3, 2, sdf, soff, f2x, f2y, dx, st, t);
-            if (sum_springs && s2 == S_FORCE) spring_sample(u_acc, w_acc, t, dx, f2x, st);
+            const bool row = __any_sync(FULL, big);
+            careful = row || big_above;
+            big_above = row;
         }
 
         // 3. gather + integrate the owned particle (gx, y)
@@ -412,13 +447,13 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
             float Ff[2];  // F as floats (sample statistics without FP64 work)
             ff Fx;        // F_x as a double-float (the grip reaction)
             if constexpr (PREC == LSM_PREC_DF) {
-                ax.add(f1x);
-                ax.add(f2x);
-                ay.add(f1y);
-                ay.add(f2y);
-                if constexpr (LAT == 0) {
-                    ax.add(f3x);
-                    ay.add(f3y);
+                DfSum ax, ay;
+                if (!careful) {
+                    ax = strip_sum<DfSum, LAT>(i3x, i2x, i1x, i0x, f0x, f1x, f2x, f3x);
+                    ay = strip_sum<DfSum, LAT>(i3y, i2y, i1y, i0y, f0y, f1y, f2y, f3y);
+                } else {
+                    ax = strip_sum<DfSumCareful, LAT>(i3x, i2x, i1x, i0x, f0x, f1x, f2x, f3x);
+                    ay = strip_sum<DfSumCareful, LAT>(i3y, i2y, i1y, i0y, f0y, f1y, f2y, f3y);
                 }
                 F[0] = ax.value(A.df_bias);
                 F[1] = ay.value(A.df_bias);
@@ -426,6 +461,14 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
                 Ff[1] = __fmul_rn(__fadd_rn(ay.hs, ay.el), A.p24);
                 Fx = ff{ax.hs, ax.el};  // (in those units)
             } else {
+                float sx_, sy_;
+                if constexpr (LAT == 0) {
+                    sx_ = f0x - i3x;
+                    sy_ = f0y - i3y;
+                } else {
+                    sx_ = f0x - i2x;
+                    sy_ = f0y - i2y;
+                }
                 if constexpr (LAT == 0) {
                     sx_ += f1x - i2x;
                     sy_ += f1y - i2y;

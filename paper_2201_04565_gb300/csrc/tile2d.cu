@@ -156,6 +156,8 @@ static TileArgs tile_args(Ctx &c)
     A.p24 = ldexpf(1.0f, 24 - c.fix_S);
     A.p0 = ldexpf(1.0f, -c.fix_S);
     A.df_bias = (unsigned)(896 + 24 - c.fix_S) << 20;
+    A.df_M = (float)std::ldexp(1.5 * c.df.unit, 23 + c.fix_S - 24);
+    A.df_cmax = (float)c.df.cmax;
     A.dt = c.h.dt;
     A.hdt = 0.5 * c.h.dt;
     A.gamma = c.h.damping;

@@ -2,7 +2,7 @@
 // second neighbours, 18 springs per interior particle) in the fixed-point
 // modes (F32, DF).
 //
-// A CTA (512 threads) owns a 32 x 8 x 8 block of voxels. Per time step it
+// A CTA (256 threads) owns a 16 x 8 x 8 block of voxels. Per time step it
 //   1. loads the block plus a one-voxel halo (phase, broken flags, positions
 //      drifted by dt vh, Eq. 3) into shared memory as 64-bit fixed point;
 //   2. compacts the block's particles into a list in raster order (porous
@@ -24,6 +24,7 @@
 // Broken flags: 9 bits per voxel (its forward springs in slot order, the
 // canonical order of the targets), written only by the owning thread; break
 // steps [9][nv].
+#include "df_pair.cuh"
 #include "tile_body.cuh"
 
 #include <algorithm>
@@ -34,8 +35,14 @@ namespace lsm {
 
 namespace {
 
-constexpr int T3X = 32, T3Y = 8, T3Z = 8, T3V = T3X * T3Y * T3Z;  // voxels per block
-constexpr int T3N = 512;                                             // threads per CTA
+// 16 x 8 x 8 blocks, four CTAs of 256 threads per SM (51 KB and 64 registers each):
+// one CTA's region load runs beside the others' springs. Against 32 x 8 x 8 blocks
+// in two CTAs of 512 the halo is a little dearer (1.76 region voxels per voxel,
+// 1.66) and the 256^3 foam's step 830 -> 775 us; 32 x 8 x 4 in three of 256: 816;
+// 16 x 8 x 4 in six of 128: 794.
+constexpr int T3X = 16, T3Y = 8, T3Z = 8, T3V = T3X * T3Y * T3Z;  // voxels per block
+constexpr int T3N = 256;                                           // threads per CTA
+constexpr int T3MIN = 4;                                           // CTAs per SM
 constexpr int R3X = T3X + 2, R3Y = T3Y + 2, R3Z = T3Z + 2, R3N = R3X * R3Y * R3Z;
 
 // shared memory of one CTA (dynamic)
@@ -75,6 +82,8 @@ struct Tile3Args {
     int ssh[9];     // their shells (1: face, 2: edge diagonal)
     float oo2[2];   // |o|^2 per shell as floats (F32 mode)
     float fa;       // lattice spacing as a float (F32 mode)
+    unsigned df_bias;     // DF: as TileArgs
+    float df_M, df_cmax;
 };
 
 // x of a grip at the strain of the step being computed (constant strain
@@ -87,34 +96,45 @@ __device__ __forceinline__ double rate_grip_x(const Tile3Args &A, int gx)
     return __dadd_rn(X, __dmul_rn(eps, __dsub_rn(X, A.xc)));
 }
 
+// A region voxel on its way from memory to shared memory (g < 0: outside).
+struct RawVoxel {
+    int64_t g;
+    uint8_t ph;
+};
+
+__device__ __forceinline__ RawVoxel voxel_at(const Tile3Args &A, int x0, int y0, int z0, int e)
+{
+    const int gx = x0 - 1 + e % R3X, gy = y0 - 1 + (e / R3X) % R3Y, gz = z0 - 1 + e / (R3X * R3Y);
+    RawVoxel r{-1, 0};
+    if (gx >= 0 && gx < A.nx && gy >= 0 && gy < A.ny && gz >= 0 && gz < A.nz) {
+        r.g = gx + (int64_t)A.nx * (gy + (int64_t)A.ny * gz);
+        r.ph = A.phase[r.g];
+    }
+    return r;
+}
+
 // rate_l, rate_r: the grips' x under the constant strain rate (RATE)
 template <int MODE, bool RATE>
-__device__ __forceinline__ void load_voxel(const Tile3Args &A, int x0, int y0, int z0, int rx, int ry, int rz,
-                                           Smem3 &S, bool &over, double rate_l, double rate_r)
+__device__ __forceinline__ void load_voxel(const Tile3Args &A, int x0, int e, const RawVoxel &r, Smem3 &S, bool &over,
+                                           double rate_l, double rate_r)
 {
-    const int gx = x0 - 1 + rx, gy = y0 - 1 + ry, gz = z0 - 1 + rz;
-    const int e = rx + R3X * (ry + R3Y * rz);
-    uint8_t ph = 0;
     uint16_t mk = 0;
     double px[3] = {0.0, 0.0, 0.0};
-    if (gx >= 0 && gx < A.nx && gy >= 0 && gy < A.ny && gz >= 0 && gz < A.nz) {
-        const int64_t g = gx + (int64_t)A.nx * (gy + (int64_t)A.ny * gz);
-        ph = A.phase[g];
-        if (ph) {
-            mk = A.mask[g];
-            const bool grip = gx == 0 || gx == A.nx - 1;
+    if (r.ph) {
+        const int gx = x0 - 1 + e % R3X;
+        mk = A.mask[r.g];
+        const bool grip = gx == 0 || gx == A.nx - 1;
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                px[c] = A.x_in[c * A.nv + g];
-                const bool fixed = grip && (c == 0 || A.grip_mode == 1);
-                if (MODE == T_STEP && !fixed) px[c] = fma(A.dt, A.vh_in[c * A.nv + g], px[c]);
-            }
-            if (RATE && MODE == T_STEP && grip) px[0] = gx == 0 ? rate_l : rate_r;
+        for (int c = 0; c < 3; c++) {
+            px[c] = A.x_in[c * A.nv + r.g];
+            const bool fixed = grip && (c == 0 || A.grip_mode == 1);
+            if (MODE == T_STEP && !fixed) px[c] = fma(A.dt, A.vh_in[c * A.nv + r.g], px[c]);
         }
-    }
+        if (RATE && MODE == T_STEP && grip) px[0] = gx == 0 ? rate_l : rate_r;
 #pragma unroll
-    for (int c = 0; c < 3; c++) S.xf[c][e] = dbl_to_fix(px[c], A.S, over);
-    S.ph[e] = ph;
+        for (int c = 0; c < 3; c++) S.xf[c][e] = dbl_to_fix(px[c], A.S, over);
+    }
+    S.ph[e] = r.ph;
     S.mk[e] = mk;
 }
 
@@ -124,21 +144,21 @@ template <int PREC, bool TEST>
 __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl, const long long *du, int s,
                                         const TypeDF &t, ff *f, ff &w, ff &u, bool sample)
 {
-    if constexpr (PREC == LSM_PREC_DF) {
+    if constexpr (PREC == LSM_PREC_DF) {  // lengths in units of 2^(24-S), as spring_df
         ff d[3];
 #pragma unroll
-        for (int c = 0; c < 3; c++) d[c] = fix_to_ff_i2f2(du[c] - dl[c], A.p24, A.p0);
+        for (int c = 0; c < 3; c++) d[c] = fix_to_ff_u24(du[c] - dl[c]);
         const ff r2 = ff_norm3_un(d[0], d[1], d[2]);
         if (TEST && ff_gt_un(r2, t.rc2)) return false;
         ff y;
         const ff g = ff_spring_g(r2, t.r0, sample ? &y : nullptr);
-        const ff cc = ff_mul_un(t.k, g);  // unnormalised: only multiplied or summed further
+        const ff cc = ff_mul_un(t.k, g);  // unnormalised: only multiplied further
 #pragma unroll
-        for (int c = 0; c < 3; c++) f[c] = ff_mul_un(cc, d[c]);
+        for (int c = 0; c < 3; c++) f[c] = ff_mul_split(cc, d[c], A.df_M);
         if (sample) {  // double-float sums: no FP64 pipe work per spring
             const ff st = ff_mul(ff_mul(r2, y), g);  // r - r0
             u = ff_add_sloppy(u, ff_mul(ff_mul_f(t.k, 0.5f), ff_sqr(st)));
-            w = ff_add_sloppy(w, ff_mul(d[0], f[0]));
+            w = ff_add_sloppy(w, ff_mul(d[0], df_pair(f[0])));
         }
     } else {  // F32: e = d - o exact, (2 o + e).e carries no cancellation
         float e[3], dd[3], num = t.cor.hi;
@@ -156,19 +176,61 @@ __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl,
         const float st = __fdividef(num, fmaf(r2f, ir, t.r0.hi));  // r - r0
         const float cc = t.k.hi * st * ir;
 #pragma unroll
-        for (int c = 0; c < 3; c++) f[c] = ff{cc * dd[c], 0.0f};
+        for (int c = 0; c < 3; c++) f[c] = ff{-(cc * dd[c]), 0.0f};  // in the form of a split force
         if (sample) {
             u = ff_add_f(u, 0.5f * t.k.hi * st * st);
-            w = ff_add_f(w, dd[0] * f[0].hi);
+            w = ff_add_f(w, dd[0] * -f[0].hi);
         }
     }
     return true;
 }
 
+// The 18 springs of a particle, DF: forces into F (split sums), new breaks of its
+// forward springs into newb; slot s's incoming spring is broken by its source's
+// flags or its own break test, which the source's thread records.
+template <typename SUM, bool TEST>
+__device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, const TypeDF *sdf, const int *soff,
+                                            int ep, int pp, uint16_t mk, const long long (&xp)[3], DfSumCareful (&F)[3],
+                                            uint16_t &newb, bool &big)
+{
+    SUM sum[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) sum[c].hs = sum[c].el = 0.0f;
+#pragma unroll 1
+    for (int s = 0; s < 9; s++) {
+        const int o = soff[s], ei = ep - o, eo = ep + o, sh = A.ssh[s] - 1;
+        const int pi = S.ph[ei], po = S.ph[eo];
+        const bool live[2] = {pi && !((S.mk[ei] >> s) & 1), po && !((mk >> s) & 1)};
+        if (!live[0] && !live[1]) continue;
+        const TypeDF &ti = sdf[live[0] ? (((pi - 1) * A.nphase) + (pp - 1)) * 2 + sh : 0];
+        const TypeDF &to = sdf[live[1] ? (((pp - 1) * A.nphase) + (po - 1)) * 2 + sh : 0];
+        long long d[3][2];
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            d[c][0] = xp[c] - S.xf[c][ei];
+            d[c][1] = S.xf[c][eo] - xp[c];
+        }
+        ff f[3][2];
+        bool brk[2];
+        spring_df_pair<3>(d, ti, to, live, A.df_M, A.df_cmax, f, brk, big);
+        if (TEST && brk[1]) newb |= (uint16_t)(1u << s);
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            sum[c].sub(f[c][0]);
+            sum[c].add(f[c][1]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        F[c].hs = sum[c].hs;
+        F[c].el = sum[c].el;
+    }
+}
+
 // RATE: constant strain-rate loading (a separate instance, so that the
 // ordinary step carries none of its code)
 template <int PREC, int MODE, bool SAMPLE, bool RATE>
-__global__ void __launch_bounds__(T3N)
+__global__ void __launch_bounds__(T3N, T3MIN)
 k_tile3d(Tile3Args A)
 {
     extern __shared__ __align__(16) unsigned char smem3[];
@@ -177,7 +239,7 @@ k_tile3d(Tile3Args A)
     __shared__ Coef4 scoef[8];
     __shared__ float smassf[8];
     __shared__ int soff[9];
-    __shared__ int wcount[T3V / 32];  // particles per 32-voxel row, then the rows' offsets
+    __shared__ int wcount[T3V / 32];  // particles per 32 voxels in block order, then the offsets
     __shared__ int ntotal;
     __shared__ double sred[T3N / 32];
 
@@ -200,9 +262,19 @@ k_tile3d(Tile3Args A)
         rate_l = rate_grip_x(A, 0);
         rate_r = rate_grip_x(A, A.nx - 1);
     }
-    for (int e = tid; e < R3N; e += T3N) {
-        const int rx = e % R3X, ry = (e / R3X) % R3Y, rz = e / (R3X * R3Y);
-        load_voxel<MODE, RATE>(A, x0, y0, z0, rx, ry, rz, S, over, rate_l, rate_r);
+    // the phases of all of a thread's voxels first, so that the loads that
+    // depend on them wait once
+    constexpr int KL = (R3N + T3N - 1) / T3N;
+    RawVoxel raw[KL];
+#pragma unroll
+    for (int k = 0; k < KL; k++) {
+        const int e = tid + k * T3N;
+        raw[k] = e < R3N ? voxel_at(A, x0, y0, z0, e) : RawVoxel{-1, 0};
+    }
+#pragma unroll
+    for (int k = 0; k < KL; k++) {
+        const int e = tid + k * T3N;
+        if (e < R3N) load_voxel<MODE, RATE>(A, x0, e, raw[k], S, over, rate_l, rate_r);
     }
     if (over) atomicOr(A.status, 2);
     __syncthreads();
@@ -210,9 +282,9 @@ k_tile3d(Tile3Args A)
     // 2. compact the block's particles (rows of 32 voxels; deterministic order:
     // raster order of the block) so that every warp works on particles
     for (int r = tid >> 5; r < T3V / 32; r += T3N / 32) {
-        const int ly = r % T3Y, lz = r / T3Y;
-        const int ep = (lane + 1) + R3X * ((ly + 1) + R3Y * (lz + 1));
-        const bool live = x0 + lane < A.nx && y0 + ly < A.ny && z0 + lz < A.nz && S.ph[ep];
+        const int l = r * 32 + lane, lx = l % T3X, ly = (l / T3X) % T3Y, lz = l / (T3X * T3Y);
+        const int ep = (lx + 1) + R3X * ((ly + 1) + R3Y * (lz + 1));
+        const bool live = x0 + lx < A.nx && y0 + ly < A.ny && z0 + lz < A.nz && S.ph[ep];
         const unsigned b = __ballot_sync(0xffffffffu, live);
         if (lane == 0) wcount[r] = __popc(b);
     }
@@ -228,9 +300,9 @@ k_tile3d(Tile3Args A)
     }
     __syncthreads();
     for (int r = tid >> 5; r < T3V / 32; r += T3N / 32) {
-        const int ly = r % T3Y, lz = r / T3Y;
-        const int ep = (lane + 1) + R3X * ((ly + 1) + R3Y * (lz + 1));
-        const bool live = x0 + lane < A.nx && y0 + ly < A.ny && z0 + lz < A.nz && S.ph[ep];
+        const int l = r * 32 + lane, lx = l % T3X, ly = (l / T3X) % T3Y, lz = l / (T3X * T3Y);
+        const int ep = (lx + 1) + R3X * ((ly + 1) + R3Y * (lz + 1));
+        const bool live = x0 + lx < A.nx && y0 + ly < A.ny && z0 + lz < A.nz && S.ph[ep];
         const unsigned b = __ballot_sync(0xffffffffu, live);
         if (live) S.list[wcount[r] + __popc(b & ((1u << lane) - 1u))] = (uint16_t)ep;
     }
@@ -250,7 +322,6 @@ k_tile3d(Tile3Args A)
         const int pp = S.ph[ep];
         const uint16_t mk = S.mk[ep];
         const long long xp[3] = {S.xf[0][ep], S.xf[1][ep], S.xf[2][ep]};
-        float hs[3] = {0.0f, 0.0f, 0.0f}, el[3] = {0.0f, 0.0f, 0.0f};
         // time steps without a sample issue the integration's global loads
         // here, so their latency hides behind the springs (the sample
         // instance keeps them late: it has no registers to spare)
@@ -263,46 +334,58 @@ k_tile3d(Tile3Args A)
                 vpre[c] = A.vh_in[c * A.nv + g];
             }
         }
-        // incoming: source p - o_s, ascending source = descending slot
-#pragma unroll 1
-        for (int s = 8; s >= 0; s--) {
-            const int eq = ep - soff[s];
-            const int pq = S.ph[eq];
-            if (!pq || ((S.mk[eq] >> s) & 1)) continue;
-            const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
-            const TypeDF t = sdf[(((pq - 1) * A.nphase) + (pp - 1)) * 2 + (A.ssh[s] - 1)];
-            ff f[3], wd{0.0f, 0.0f}, ud{0.0f, 0.0f};
-            if (!spring3<PREC, MODE == T_STEP>(A, xq, xp, s, t, f, wd, ud, false)) continue;
+        // one spring at a time (sample steps, and F32, whose forces are plain
+        // floats: hi alone) the sums keep their errors
+        DfSumCareful F3[3];
 #pragma unroll
-            for (int c = 0; c < 3; c++) {  // F -= f (cascaded sum)
-                const ff tt = two_sum(hs[c], -f[c].hi);
-                hs[c] = tt.hi;
-                el[c] = __fadd_rn(el[c], __fsub_rn(tt.lo, f[c].lo));
+        for (int c = 0; c < 3; c++) F3[c].hs = F3[c].el = 0.0f;
+        uint16_t newb = 0;
+        if constexpr (PREC == LSM_PREC_DF && !SAMPLE) {
+            // a slot's incoming (source p - o_s) and outgoing (target p + o_s)
+            // springs side by side on packed instructions
+            bool big = false;
+            tile3_pairs<DfSum, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
+            if (big) {  // a force beyond the split's exact range: the sums again, with their errors
+                newb = 0;
+                tile3_pairs<DfSumCareful, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
+            }
+        } else {
+            // incoming by ascending source (descending slot), then outgoing
+#pragma unroll 1
+            for (int s = 8; s >= 0; s--) {
+                const int eq = ep - soff[s];
+                const int pq = S.ph[eq];
+                if (!pq || ((S.mk[eq] >> s) & 1)) continue;
+                const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
+                const TypeDF t = sdf[(((pq - 1) * A.nphase) + (pp - 1)) * 2 + (A.ssh[s] - 1)];
+                ff f[3], wd{0.0f, 0.0f}, ud{0.0f, 0.0f};
+                if (!spring3<PREC, MODE == T_STEP>(A, xq, xp, s, t, f, wd, ud, false)) continue;
+#pragma unroll
+                for (int c = 0; c < 3; c++) F3[c].sub(f[c]);
+            }
+#pragma unroll 1
+            for (int s = 0; s < 9; s++) {
+                const int eq = ep + soff[s];
+                const int pq = S.ph[eq];
+                if (!pq || ((mk >> s) & 1)) continue;
+                const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
+                const TypeDF t = sdf[(((pp - 1) * A.nphase) + (pq - 1)) * 2 + (A.ssh[s] - 1)];
+                ff f[3];
+                if (!spring3<PREC, MODE == T_STEP>(A, xp, xq, s, t, f, w_acc, u_acc, SAMPLE)) {
+                    newb |= (uint16_t)(1u << s);
+                    continue;
+                }
+#pragma unroll
+                for (int c = 0; c < 3; c++) F3[c].add(f[c]);
             }
         }
-        // outgoing: target p + o_s, ascending slot
-        uint16_t newb = 0;
-#pragma unroll 1
-        for (int s = 0; s < 9; s++) {
-            const int eq = ep + soff[s];
-            const int pq = S.ph[eq];
-            if (!pq || ((mk >> s) & 1)) continue;
-            const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
-            const TypeDF t = sdf[(((pp - 1) * A.nphase) + (pq - 1)) * 2 + (A.ssh[s] - 1)];
-            ff f[3];
-            if (!spring3<PREC, MODE == T_STEP>(A, xp, xq, s, t, f, w_acc, u_acc, SAMPLE)) {
-                newb |= (uint16_t)(1u << s);
-                A.brk[(int64_t)s * A.nv + g] = step_now;
-                atomicMin(A.first_break, (unsigned long long)step_now);
-                atomicAdd(A.nbroken, 1ull);
-                continue;
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) {  // F += f
-                const ff tt = two_sum(hs[c], f[c].hi);
-                hs[c] = tt.hi;
-                el[c] = __fadd_rn(el[c], __fadd_rn(tt.lo, f[c].lo));
-            }
+        if (MODE == T_STEP && newb) {
+            for (int s = 0; s < 9; s++)
+                if ((newb >> s) & 1) {
+                    A.brk[(int64_t)s * A.nv + g] = step_now;
+                    atomicMin(A.first_break, (unsigned long long)step_now);
+                    atomicAdd(A.nbroken, 1ull);
+                }
         }
         if (MODE == T_STEP && newb) A.mask[g] = (uint16_t)(mk | newb);
 
@@ -310,13 +393,14 @@ k_tile3d(Tile3Args A)
         // the region load (same operations on the same inputs)
         const bool grip = gx == 0 || gx == A.nx - 1;
         const int ph = pp - 1;
-        if (SAMPLE && gx == A.nx - 1) reactf = ff_add_sloppy(reactf, ff{-hs[0], -el[0]});
+        if (SAMPLE && gx == A.nx - 1) reactf = ff_add_sloppy(reactf, ff{-F3[0].hs, -F3[0].el});
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             const bool fixed = grip && (c == 0 || A.grip_mode == 1);
             const int64_t q = c * A.nv + g;
-            const double F = f2d_force(hs[c]) + f2d_force(el[c]);
-            const float Ff = __fadd_rn(hs[c], el[c]);
+            const double F = F3[c].value(A.df_bias);
+            float Ff = __fadd_rn(F3[c].hs, F3[c].el);
+            if (PREC == LSM_PREC_DF) Ff = __fmul_rn(Ff, A.p24);  // back from units of 2^(24-S)
             double xr;
             double vh;
             if constexpr (PRE) {
@@ -369,11 +453,12 @@ k_tile3d(Tile3Args A)
         const double t4 = bsum_ff<T3N / 32>(reactf, sred);
         const double t5 = bmax_f<T3N / 32>(resf, sred);
         if (tid == 0) {
-            A.part_s[tile_id] = t0;
-            A.part_s[A.ntiles + tile_id] = t1;
+            const double u = PREC == LSM_PREC_DF ? (double)A.p24 : 1.0;  // from units of 2^(24-S) (exact)
+            A.part_s[tile_id] = t0 * (u * u);
+            A.part_s[A.ntiles + tile_id] = t1 * (u * u);
             A.part_p[tile_id] = t2;
             A.part_p[A.ntiles + tile_id] = t3;
-            A.part_p[2 * A.ntiles + tile_id] = t4;
+            A.part_p[2 * A.ntiles + tile_id] = t4 * u;
             A.part_p[3 * A.ntiles + tile_id] = t5;
         }
     }
@@ -448,6 +533,9 @@ Tile3Args tile3_args(Ctx &c)
         A.ssh[s] = l2;
     }
     A.fa = (float)aa;
+    A.df_bias = (unsigned)(896 + (c.h.precision == LSM_PREC_DF ? 24 - c.fix_S : 0)) << 20;
+    A.df_M = (float)std::ldexp(1.5 * c.df.unit, 23 + c.fix_S - 24);
+    A.df_cmax = (float)c.df.cmax;
     A.oo2[0] = (float)(aa * aa);
     A.oo2[1] = (float)(2.0 * aa * aa);
     return A;
@@ -531,6 +619,7 @@ cudaError_t tile3_upload(Ctx &c)
     c.fix_S = std::min(c.fix_S, 47 - (int)std::ceil(std::log2(h.a * std::sqrt(2.0))));
     c.fix_S = std::min(c.fix_S, 47 - (int)std::floor(std::log2(max_critical_length(h.types))));
     c.a_fix = std::llround(std::ldexp(h.a, c.fix_S));
+    c.df = df_split(h.types, 18);
     const double aa = std::ldexp((double)c.a_fix, -c.fix_S);
     std::vector<TypeDF> tdf(h.types.size());
     for (size_t q = 0; q < h.types.size(); q++) {
@@ -538,9 +627,11 @@ cudaError_t tile3_upload(Ctx &c)
         const double shell = (q & 1) ? 2.0 : 1.0;
         const double p = t.r0 * t.r0, pe = std::fma(t.r0, t.r0, -p);
         const double o2 = shell * aa * aa, o2e = shell * std::fma(aa, aa, -(aa * aa));
+        // DF: lengths in units of 2^(24-S) (exact power-of-two scaling)
+        const double ul = h.precision == LSM_PREC_DF ? std::ldexp(1.0, c.fix_S - 24) : 1.0;
         tdf[q].k = split_ff3(t.k);
-        tdf[q].r0 = split_ff3(t.r0);
-        tdf[q].rc2 = split_ff3(t.rc2);
+        tdf[q].r0 = split_ff3(t.r0 * ul);
+        tdf[q].rc2 = split_ff3(t.rc2 * ul * ul);
         tdf[q].cor = split_ff3((o2 - p) + (o2e - pe));
     }
     std::vector<int64_t> sbase(nv, 0);

@@ -7,6 +7,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "df_pair.cuh"
 #include "dfloat.cuh"
 #include "exact64.cuh"
 #include "lsm_internal.h"
@@ -116,6 +117,7 @@ struct TileArgs {
     double hrow;               // triangular packing: row height
     float p24, p0;             // 2^(24-S), 2^-S
     unsigned df_bias;          // DF: f2d_force_scaled bias for forces held in units of p24
+    float df_M, df_cmax;       // DF: the force split's 1.5 2^23 u (in those units), and the c it is exact for
     double dt, hdt, gamma, a;
     int grip_mode;
     int rate_on;               // constant strain rate: grips at rate_eps0 + (s - rate_step0) rate_dt
@@ -145,35 +147,72 @@ __host__ __device__ constexpr int tile_min_ctas()
                                      : 6;
 }
 
-// Cascaded double-float sum (Ogita, Rump and Oishi, 2005) of a particle's
-// spring forces in the canonical order: a TwoSum chain over the high parts,
-// with their errors and the low parts summed in float. value() is the sum
-// as a double (exact conversion of both parts, one FP64 addition).
+// Sum of a particle's DF spring forces in the canonical order. A force is held
+// split (ff_mul_split): f = lo - hi, hi a multiple of the context's unit u. While
+// every |hi| is within the split's range (df_split), the sums of all of them are
+// exact in float, and the low parts, below u, are summed in float beside them: two
+// additions per term (DfSum). A spring compressed beyond that (the springs'
+// "big" flag) takes the cascaded sum (Ogita, Rump and Oishi, 2005) of the same
+// terms, a TwoSum chain over the high parts (DfSumCareful): where no high sum
+// rounds, its errors are 0 and both give the same bits, so kernels may decide
+// it per warp, per block or always. value(): the sum as a double (exact
+// conversion of both parts, one FP64 addition; bias: the unit the terms are
+// held in, f2d_force_scaled).
 struct DfSum {
     float hs, el;
     __device__ __forceinline__ void first_neg(ff t)
     {
-        hs = -t.hi;
+        hs = t.hi;
         el = -t.lo;
     }
     __device__ __forceinline__ void sub(ff o)
     {
-        const ff t = two_sum(hs, -o.hi);
-        hs = t.hi;
-        el = __fadd_rn(el, __fsub_rn(t.lo, o.lo));
+        hs = __fadd_rn(hs, o.hi);
+        el = __fsub_rn(el, o.lo);
     }
     __device__ __forceinline__ void add(ff o)
     {
-        const ff t = two_sum(hs, o.hi);
-        hs = t.hi;
-        el = __fadd_rn(el, __fadd_rn(t.lo, o.lo));
+        hs = __fsub_rn(hs, o.hi);
+        el = __fadd_rn(el, o.lo);
     }
-    // the sum as a double; bias: the unit the terms are held in (f2d_force_scaled)
     __device__ __forceinline__ double value(unsigned bias) const
     {
         return f2d_force_scaled(hs, bias) + f2d_force_scaled(el, bias);
     }
 };
+
+struct DfSumCareful : DfSum {
+    __device__ __forceinline__ void sub(ff o)
+    {
+        const ff t = two_sum(hs, o.hi);
+        hs = t.hi;
+        el = __fadd_rn(el, __fsub_rn(t.lo, o.lo));
+    }
+    __device__ __forceinline__ void add(ff o)
+    {
+        const ff t = two_sum(hs, -o.hi);
+        hs = t.hi;
+        el = __fadd_rn(el, __fadd_rn(t.lo, o.lo));
+    }
+};
+
+// The canonical order of a square-lattice particle: incoming slots 3, 2, 1, 0, then
+// its own, o[0], o[stride], ...
+template <typename SUM>
+__device__ __forceinline__ DfSum df_gather(ff i3, ff i2, ff i1, ff i0, const ff *o, int stride)
+{
+    SUM acc;
+    acc.first_neg(i3);
+    acc.sub(i2);
+    acc.sub(i1);
+    acc.sub(i0);
+#pragma unroll
+    for (int sl = 0; sl < 4; sl++) acc.add(o[sl * stride]);
+    return acc;
+}
+
+// A split force as an ordinary pair (sample sums).
+__device__ __forceinline__ ff df_pair(ff f) { return ff{-f.hi, f.lo}; }
 
 // The fixed-point modes' spring arithmetic, shared by every 2D kernel that
 // evaluates springs (tile, strip and batched kernels), so that all of them
@@ -181,8 +220,8 @@ struct DfSum {
 // (dxq, dyq) = x_q - x_p of an intact spring of type t in forward slot
 // `slot`. Returns true when the break test (TEST) fires: r^2 > rc^2, the
 // force is then left at zero. Otherwise writes the force on the lower
-// endpoint, f = k (1 - r0/r) d (Eq. 2), and with SAMPLE the spring's x
-// component d_x and its stretch r - r0.
+// endpoint, f = k (1 - r0/r) d (Eq. 2; DF: split, see DfSum), and with SAMPLE the
+// spring's x component d_x and its stretch r - r0.
 
 // Double-float force: d as a double-float (two exact 24-bit chunks), 1/r by
 // one double-float Newton step, k (r - r0) / r = k (1 - r0 / r). Lengths are
@@ -191,7 +230,7 @@ struct DfSum {
 // unit too: exactly the unscaled values times 2^(S-24).
 template <bool TEST, bool SAMPLE>
 __device__ __forceinline__ bool spring_df(long long dxq, long long dyq, const TypeDF &t, const TileArgs &A,
-                                          ff &fx, ff &fy, ff &dx, ff &st)
+                                          ff &fx, ff &fy, ff &dx, ff &st, bool &big)
 {
     const ff dxf = fix_to_ff_u24(dxq);
     const ff dyf = fix_to_ff_u24(dyq);
@@ -199,9 +238,10 @@ __device__ __forceinline__ bool spring_df(long long dxq, long long dyq, const Ty
     if (TEST && ff_gt_un(r2, t.rc2)) return true;
     ff y;
     const ff g = ff_spring_g(r2, t.r0, SAMPLE ? &y : nullptr);
-    const ff c = ff_mul_un(t.k, g);  // the products stay unnormalised: they are only
-    fx = ff_mul_un(c, dxf);          // multiplied or summed further (DfSum)
-    fy = ff_mul_un(c, dyf);
+    const ff c = ff_mul_un(t.k, g);  // unnormalised: only multiplied further
+    big |= fabsf(c.hi) > A.df_cmax;
+    fx = ff_mul_split(c, dxf, A.df_M);
+    fy = ff_mul_split(c, dyf, A.df_M);
     if (SAMPLE) {
         dx = dxf;
         st = ff_mul(ff_mul(r2, y), g);  // r - r0
@@ -261,7 +301,7 @@ __device__ __forceinline__ void eval_spring(const TileArgs &A, int rp, int rq, i
                                             const uint8_t *sph, const uint8_t *smk, FT *sf,
                                             const SpringType *stab, const TypeDF *sdf, const ff (*soff)[3],
                                             int *snew, int64_t gsrc, long long step_now, AT &w_acc,
-                                            AT &u_acc)
+                                            AT &u_acc, bool &big)
 {
     FT fx{}, fy{};
     const uint8_t pp = sph[rp], pq = sph[rq];
@@ -297,10 +337,10 @@ __device__ __forceinline__ void eval_spring(const TileArgs &A, int rp, int rq, i
             } else {  // LSM_PREC_DF
                 ff dxf, st;
                 brk_now = spring_df<MODE == T_STEP, SAMPLE && OWNER>(sxf[rq] - sxf[rp], syf[rq] - syf[rp], t, A,
-                                                                     fx, fy, dxf, st);
+                                                                     fx, fy, dxf, st, big);
                 if (SAMPLE && OWNER && !brk_now) {  // double-float sums: no FP64 pipe work per spring
                     u_acc = ff_add_sloppy(u_acc, ff_mul(ff_mul_f(t.k, 0.5f), ff_sqr(st)));
-                    w_acc = ff_add_sloppy(w_acc, ff_mul(dxf, fx));
+                    w_acc = ff_add_sloppy(w_acc, ff_mul(dxf, df_pair(fx)));
                 }
             }
         }
@@ -313,6 +353,44 @@ __device__ __forceinline__ void eval_spring(const TileArgs &A, int rp, int rq, i
     }
     sf[(0 * 4 + slot) * NS + rp] = fx;
     sf[(1 * 4 + slot) * NS + rp] = fy;
+}
+
+// Two forward springs (slots sa, sb of one shell) of an owned pixel, DF time steps
+// without a sample, side by side (df_pair.cuh; the bits of eval_spring).
+template <int NS>
+__device__ __forceinline__ void eval_pair(const TileArgs &A, int rp, int sa, int sb, int oa, int ob,
+                                          const long long *sxf, const long long *syf, const uint8_t *sph,
+                                          const uint8_t *smk, ff *sf, const TypeDF *sdf, int *snew, int64_t gsrc,
+                                          long long step_now, bool &big)
+{
+    ff f[2][2] = {};
+    const int ra = rp + oa, rb = rp + ob;
+    const int pp = sph[rp], pa = sph[ra], pb = sph[rb];
+    const unsigned mk = smk[rp];
+    const bool live[2] = {pp && pa && !((mk >> sa) & 1u), pp && pb && !((mk >> sb) & 1u)};
+    if (live[0] || live[1]) {
+        const int row = (pp - 1) * A.nphase - 1, sh = sa & 1;
+        const long long d[2][2] = {{sxf[ra] - sxf[rp], sxf[rb] - sxf[rp]}, {syf[ra] - syf[rp], syf[rb] - syf[rp]}};
+        bool brk[2];
+        spring_df_pair<2>(d, sdf[live[0] ? (row + pa) * 2 + sh : 0], sdf[live[1] ? (row + pb) * 2 + sh : 0], live,
+                          A.df_M, A.df_cmax, f, brk, big);
+        if (brk[0] || brk[1]) {
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                if (!brk[h]) continue;
+                const int slot = h ? sb : sa;
+                atomicOr(&snew[rp], 1 << slot);
+                A.brk[(int64_t)slot * A.np + gsrc] = step_now;
+                atomicMin(A.first_break, (unsigned long long)step_now);
+                atomicAdd(A.nbroken, 1ull);
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        sf[(c * 4 + sa) * NS + rp] = f[c][0];
+        sf[(c * 4 + sb) * NS + rp] = f[c][1];
+    }
 }
 
 // Constant strain rate: x of a grip in column gx at the strain of the step
@@ -465,16 +543,22 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
     // 2a. forward springs of the owned particles
     using AT = typename std::conditional<FIX, ff, double>::type;  // per-thread sample sums
     AT w_acc{}, u_acc{};
+    bool big = false;  // DF: a force beyond the split's exact range
     constexpr int dq[4] = {1, RX - 1, RX, RX + 1};
 #pragma unroll
     for (int k = 0; k < TY / NW; k++) {
         const int ry = warp + k * NW + 1, rx = lane + 1;
         const int rp = ry * RX + rx;
         const int64_t g = (int64_t)(y0 + ry - 1) * A.nx + (x0 + lane);
+        if constexpr (PREC == LSM_PREC_DF && MODE == T_STEP && !SAMPLE) {
+            eval_pair<NS>(A, rp, 0, 2, dq[0], dq[2], sxf, syf, sph, smk, sf, sdf, snew, g, step_now, big);
+            eval_pair<NS>(A, rp, 1, 3, dq[1], dq[3], sxf, syf, sph, smk, sf, sdf, snew, g, step_now, big);
+        } else {
 #pragma unroll
-        for (int slot = 0; slot < 4; slot++)
-            eval_spring<PREC, MODE, SAMPLE, true, NR, NS>(A, rp, rp + dq[slot], slot, sx, sy, sxf, syf, sph, smk,
-                                                          sf, stab, sdf, soff, snew, g, step_now, w_acc, u_acc);
+            for (int slot = 0; slot < 4; slot++)
+                eval_spring<PREC, MODE, SAMPLE, true, NR, NS>(A, rp, rp + dq[slot], slot, sx, sy, sxf, syf, sph, smk,
+                                                              sf, stab, sdf, soff, snew, g, step_now, w_acc, u_acc, big);
+        }
     }
     // 2b. springs from halo sources into the tile (also evaluated, with the
     // same result, by the tile that owns their lower endpoint)
@@ -495,9 +579,11 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
         }
         const int rp = ry * RX + rx;
         eval_spring<PREC, MODE, SAMPLE, false, NR, NS>(A, rp, rp + dq[slot], slot, sx, sy, sxf, syf, sph, smk, sf,
-                                                       stab, sdf, soff, snew, 0, step_now, w_acc, u_acc);
+                                                       stab, sdf, soff, snew, 0, step_now, w_acc, u_acc, big);
     }
-    __syncthreads();
+    bool careful = false;
+    if constexpr (PREC == LSM_PREC_DF) careful = __syncthreads_or(big);
+    else __syncthreads();
 
     // 3. gather + integrate the owned particles
     double mvx2 = 0.0, ke = 0.0, react = 0.0, res = 0.0;
@@ -532,16 +618,13 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
                 F[c] = acc;
             }
         } else if constexpr (PREC == LSM_PREC_DF) {
-            // cascaded summation in the fixed order above (DfSum)
 #pragma unroll
             for (int c = 0; c < 2; c++) {
+                const ff i3 = sf[(c * 4 + 3) * NS + s3], i2 = sf[(c * 4 + 2) * NS + s2], i1 = sf[(c * 4 + 1) * NS + s1],
+                         i0 = sf[(c * 4 + 0) * NS + s0];
                 DfSum acc;
-                acc.first_neg(sf[(c * 4 + 3) * NS + s3]);
-                acc.sub(sf[(c * 4 + 2) * NS + s2]);
-                acc.sub(sf[(c * 4 + 1) * NS + s1]);
-                acc.sub(sf[(c * 4 + 0) * NS + s0]);
-#pragma unroll
-                for (int sl = 0; sl < 4; sl++) acc.add(sf[(c * 4 + sl) * NS + rp]);
+                if (!careful) acc = df_gather<DfSum>(i3, i2, i1, i0, sf + c * 4 * NS + rp, NS);
+                else acc = df_gather<DfSumCareful>(i3, i2, i1, i0, sf + c * 4 * NS + rp, NS);
                 F[c] = acc.value(A.df_bias);
                 Ff[c] = __fmul_rn(__fadd_rn(acc.hs, acc.el), A.p24);  // back from units of 2^(24-S)
                 Fd[c] = ff{acc.hs, acc.el};                            // (in those units)

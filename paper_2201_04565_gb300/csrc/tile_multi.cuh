@@ -31,6 +31,7 @@
 // (tile_multi.cu) for where the lines lie.
 #pragma once
 
+#include "df_pair.cuh"
 #include "tile_body.cuh"
 
 namespace lsm {
@@ -169,6 +170,7 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
         // and dropped), so that their dependent chains overlap
         FT fx[NS], fy[NS];
         unsigned nb = 0;
+        bool big = false;  // DF: a force beyond the split's exact range
         if (ph && depth >= s) {
             unsigned live = 0, longer = 0;
             int ti[NS], qq[NS];
@@ -202,6 +204,22 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
                         w_acc += ml(dd[q][0], f[q][0]);
                     }
                 }
+            } else if constexpr (PREC == LSM_PREC_DF && !SAMPLE) {  // two springs at a time
+#pragma unroll
+                for (int q = 0; q < NS; q += 2) {
+                    const long long dd[2][2] = {{sx[qq[q]] - mx, sx[qq[q + 1]] - mx},
+                                                {sx[N + qq[q]] - my, sx[N + qq[q + 1]] - my}};
+                    const bool lv[2] = {(bool)((live >> q) & 1), (bool)((live >> (q + 1)) & 1)};
+                    ff f[2][2];
+                    bool brk[2];
+                    spring_df_pair<2>(dd, sdf[ti[q]], sdf[ti[q + 1]], lv, A.df_M, A.df_cmax, f, brk, big);
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        if (brk[h]) longer |= 1u << (q + h);
+                        fx[q + h] = f[0][h];
+                        fy[q + h] = f[1][h];
+                    }
+                }
             } else {
 #pragma unroll
                 for (int q = 0; q < NS; q++) {
@@ -213,7 +231,7 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
                             longer |= 1u << q;
                     } else {
                         if (ff_gt_un(ff_norm2_un(fix_to_ff_u24(dx), fix_to_ff_u24(dy)), t.rc2)) longer |= 1u << q;
-                        spring_df<false, SAMPLE>(dx, dy, t, A, fx[q], fy[q], dxf, st);
+                        spring_df<false, SAMPLE>(dx, dy, t, A, fx[q], fy[q], dxf, st, big);
                     }
                     if (last && own && ((live & ~longer) >> q) & 1) {
                         if constexpr (PREC == LSM_PREC_F32) {
@@ -221,7 +239,7 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
                             w_acc = ff_add_f(w_acc, dxf * fx[q]);
                         } else if constexpr (PREC == LSM_PREC_DF) {
                             u_acc = ff_add_sloppy(u_acc, ff_mul(ff_mul_f(t.k, 0.5f), ff_sqr(st)));
-                            w_acc = ff_add_sloppy(w_acc, ff_mul(dxf, fx[q]));
+                            w_acc = ff_add_sloppy(w_acc, ff_mul(dxf, df_pair(fx[q])));
                         }
                     }
                 }
@@ -257,38 +275,33 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
                     }
             }
         }
-        __syncthreads();
+        bool careful = false;
+        if constexpr (PREC == LSM_PREC_DF) careful = __syncthreads_or(big);
+        else __syncthreads();
         // gather and integrate
         if (comps && ph && depth > s) {
 #pragma unroll
             for (int c = 0; c < NC; c++) {
                 const FT *f = sf + (c0 + c) * 4 * N + e;
                 const FT i3 = f[3 * N - RX - 1], i2 = f[2 * N - RX], i1 = f[N - RX + 1], i0 = f[-1];
-                const FT o0 = f[0], o1 = f[N], o2 = f[2 * N], o3 = f[3 * N];
                 double F;
                 float Ff = 0.0f;
                 ff Fd{0.0f, 0.0f};
                 if constexpr (PREC == LSM_PREC_EXACT64) {
                     F = sb(sb(sb(sb(0.0, i3), i2), i1), i0);
-                    F = ad(ad(ad(ad(F, o0), o1), o2), o3);
+                    F = ad(ad(ad(ad(F, f[0]), f[N]), f[2 * N]), f[3 * N]);
                 } else if constexpr (PREC == LSM_PREC_DF) {
                     DfSum acc;
-                    acc.first_neg(i3);
-                    acc.sub(i2);
-                    acc.sub(i1);
-                    acc.sub(i0);
-                    acc.add(o0);
-                    acc.add(o1);
-                    acc.add(o2);
-                    acc.add(o3);
+                    if (!careful) acc = df_gather<DfSum>(i3, i2, i1, i0, f, N);
+                    else acc = df_gather<DfSumCareful>(i3, i2, i1, i0, f, N);
                     F = acc.value(A.df_bias);
                     Ff = __fmul_rn(__fadd_rn(acc.hs, acc.el), A.p24);  // back from units of 2^(24-S)
                     Fd = ff{acc.hs, acc.el};                            // (in those units)
                 } else {
-                    float acc = o0 - i3;
-                    acc += o1 - i2;
-                    acc += o2 - i1;
-                    acc += o3 - i0;
+                    float acc = f[0] - i3;
+                    acc += f[N] - i2;
+                    acc += f[2 * N] - i1;
+                    acc += f[3 * N] - i0;
                     F = f2d_force(acc);
                     Ff = acc;
                     Fd = ff{acc, 0.0f};
