@@ -33,203 +33,423 @@
 namespace lsm {
 namespace nn {
 
-// out[i] = sum over splits s (in order) of part[s][i].
-__global__ void k_fold(const float *__restrict__ part, int64_t n, int splits, float *__restrict__ out)
+// The kernels between the convolutions move activations of 16 to 64 MB that
+// mostly stay in L2, so what bounds them is the number of bytes a thread has
+// in flight: every thread handles eight channels as one 16-byte access (all
+// channel counts are multiples of 32, all slice offsets multiples of 8), and
+// the reductions over pixels run beside a pass that reads the tensor anyway.
+
+__device__ __forceinline__ uint4 ld8(const bf16 *p) { return *reinterpret_cast<const uint4 *>(p); }
+__device__ __forceinline__ void st8(bf16 *p, const uint4 &v) { *reinterpret_cast<uint4 *>(p) = v; }
+__device__ __forceinline__ unsigned word(const uint4 &v, int w) { return w == 0 ? v.x : w == 1 ? v.y : w == 2 ? v.z : v.w; }
+// channel 2 w + h of eight packed ones
+__device__ __forceinline__ float ch(const uint4 &v, int w, int h)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    return __uint_as_float(h ? word(v, w) & 0xffff0000u : word(v, w) << 16);
+}
+__device__ __forceinline__ unsigned pack2(float lo, float hi)
+{
+    return (unsigned)__bfloat16_as_ushort(__float2bfloat16(lo)) |
+           (unsigned)__bfloat16_as_ushort(__float2bfloat16(hi)) << 16;
+}
+// the two channels of a gradient word where the activation's are positive, else 0
+__device__ __forceinline__ unsigned relu_mask(unsigned g, unsigned a)
+{
+    return (__uint_as_float(a << 16) > 0.0f ? g & 0xffffu : 0u) |
+           (__uint_as_float(a & 0xffff0000u) > 0.0f ? g & 0xffff0000u : 0u);
+}
+__device__ __forceinline__ void add2(float *acc, unsigned g)
+{
+    acc[0] += __uint_as_float(g << 16);
+    acc[1] += __uint_as_float(g & 0xffff0000u);
+}
+
+// Pixel reductions: a block of 256 threads covers 32 channels (blockIdx.y) as
+// 64 pixels x 4 groups of eight; it strides over the pixels and leaves one
+// partial sum per channel, folded in a fixed order by k_fold_cols.
+constexpr int RED_PIX = 64;
+constexpr int RED_BLOCKS = 1216;  // 8 blocks on each of 152 SMs
+
+static dim3 red_grid(int64_t M, int C)
+{
+    const int chunks = C / 32;
+    const int64_t most = RED_BLOCKS / chunks > 1 ? RED_BLOCKS / chunks : 1;
+    return dim3((unsigned)std::min<int64_t>((M + RED_PIX - 1) / RED_PIX, most), (unsigned)chunks);
+}
+
+// Sum of v over the warp's eight pixels (lanes of one channel group differ in bits 2 to 4).
+__device__ __forceinline__ float pix_sum(float v)
+{
+    v += __shfl_xor_sync(0xffffffffu, v, 4);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    return v + __shfl_xor_sync(0xffffffffu, v, 16);
+}
+
+// The block's sums of its 32 channels, to part[blockIdx.x][C].
+__device__ __forceinline__ void red_store(const float acc[8], int C, float *__restrict__ part)
+{
+    __shared__ float sh[8][32];
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const float v = pix_sum(acc[k]);
+        if ((t & 31) < 4) sh[t >> 5][(t & 3) * 8 + k] = v;
+    }
+    __syncthreads();
+    if (t < 32) {
+        float s = sh[0][t];
+#pragma unroll
+        for (int w = 1; w < 8; w++) s += sh[w][t];
+        part[(int64_t)blockIdx.x * C + blockIdx.y * 32 + t] = s;
+    }
+}
+
+// Column sums of partial rows, for several segments in one launch: a block
+// folds 32 columns with 32 row lanes (rows l, l + 32, ... in order, then the
+// lanes in order).
+struct FoldSeg {
+    const float *part;
+    float *out;
+    int stride, cols, rows, first;  // row stride; columns; rows; first block
+    float scale;
+};
+constexpr int MAX_SEG = 16;
+struct FoldTab {
+    FoldSeg s[MAX_SEG];
+    int n = 0, blocks = 0;
+    void add(const float *part, int stride, int cols, int rows, float scale, float *out)
+    {
+        s[n++] = FoldSeg{part, out, stride, cols, rows, blocks, scale};
+        blocks += (cols + 31) / 32;
+    }
+};
+
+__global__ void __launch_bounds__(1024) k_fold_cols(const __grid_constant__ FoldTab tab)
+{
+    __shared__ float sh[32][33];
+    int q = 0;
+    while (q + 1 < tab.n && (int)blockIdx.x >= tab.s[q + 1].first) q++;
+    const FoldSeg &g = tab.s[q];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5, c = ((int)blockIdx.x - g.first) * 32 + lane;
     float s = 0.0f;
-    for (int q = 0; q < splits; q++) s += part[(int64_t)q * n + i];
-    out[i] = s;
+    if (c < g.cols) {
+#pragma unroll 8
+        for (int r = row; r < g.rows; r += 32) s += g.part[(int64_t)r * g.stride + c];
+    }
+    sh[row][lane] = s;
+    __syncthreads();
+    if (row == 0 && c < g.cols) {
+        s = sh[0][lane];
+#pragma unroll
+        for (int l = 1; l < 32; l++) s += sh[l][lane];
+        g.out[c] = s * g.scale;
+    }
 }
 
-// Wr[ci][tap'][co] = W[co][taps - 1 - tap'][ci]
-__global__ void k_rotate(const bf16 *__restrict__ W, bf16 *__restrict__ Wr, int Cout, int Cin, int taps)
+// Column sums of grad[M][C] (rows g_cs apart) as partial rows of C.
+__global__ void __launch_bounds__(256) k_bias_part(const bf16 *__restrict__ grad, int g_cs, int C, int64_t M,
+                                                   float *__restrict__ part)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n = (int64_t)Cout * Cin * taps;
-    if (i >= n) return;
-    const int co = (int)(i % Cout);
-    const int64_t r = i / Cout;
-    const int tp = (int)(r % taps);
-    const int ci = (int)(r / taps);
-    Wr[i] = W[((int64_t)co * taps + (taps - 1 - tp)) * Cin + ci];
+    const int t = threadIdx.x, c = blockIdx.y * 32 + (t & 3) * 8;
+    float acc[8] = {};
+#pragma unroll 4
+    for (int64_t m = (int64_t)blockIdx.x * RED_PIX + (t >> 2); m < M; m += (int64_t)gridDim.x * RED_PIX) {
+        const uint4 g = ld8(grad + m * g_cs + c);
+#pragma unroll
+        for (int w = 0; w < 4; w++) add2(acc + 2 * w, word(g, w));
+    }
+    red_store(acc, C, part);
 }
 
-cudaError_t rotate_weights(const bf16 *W, bf16 *Wr, int Cout, int Cin, int taps, cudaStream_t st)
+// Bias gradient of a convolution called by itself. The scratch holds at least
+// 32 C floats (the caller's weight partials: C rows of taps x Cin >= 32).
+cudaError_t bias_grad(const bf16 *grad, int g_cs, int C, int64_t M, float *db, float *scratch, size_t scratch_floats,
+                      cudaStream_t st)
 {
-    const int64_t n = (int64_t)Cout * Cin * taps;
-    k_rotate<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(W, Wr, Cout, Cin, taps);
+    dim3 grid = red_grid(M, C);
+    grid.x = (unsigned)std::min<size_t>(grid.x, scratch_floats / C);
+    k_bias_part<<<grid, 256, 0, st>>>(grad, g_cs, C, M, scratch);
+    FoldTab tab;
+    tab.add(scratch, C, C, (int)grid.x, 1.0f, db);
+    k_fold_cols<<<tab.blocks, 1024, 0, st>>>(tab);
     return cudaGetLastError();
+}
+
+// Wr[ci][tap'][co] = W[co][taps - 1 - tap'][ci] for every convolution that
+// passes a gradient on, in one launch: a block transposes one 32 x 32 tile of
+// one tap through shared memory. (One launch per convolution, reading along
+// co with a stride of a whole weight row, took 45 us for the 13; the pass
+// moves 7.8 MB.)
+struct RotSeg {
+    int64_t off;
+    int Cout, Cin, first;
+};
+struct RotTab {
+    RotSeg s[MAX_SEG];
+    int n = 0, blocks = 0;
+};
+
+__global__ void __launch_bounds__(256) k_rotate(const __grid_constant__ RotTab tab, const bf16 *__restrict__ W,
+                                                bf16 *__restrict__ Wr)
+{
+    __shared__ bf16 sh[32][34];
+    int q = 0;
+    while (q + 1 < tab.n && (int)blockIdx.x >= tab.s[q + 1].first) q++;
+    const int Cout = tab.s[q].Cout, Cin = tab.s[q].Cin;
+    const int64_t off = tab.s[q].off;
+    const int i = (int)blockIdx.x - tab.s[q].first, nci = Cin / 32, tap = i % 9, r = i / 9;
+    const int ci0 = (r % nci) * 32, co0 = (r / nci) * 32, lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = y; j < 32; j += 8) sh[j][lane] = W[off + ((int64_t)(co0 + j) * 9 + 8 - tap) * Cin + ci0 + lane];
+    __syncthreads();
+#pragma unroll
+    for (int j = y; j < 32; j += 8) Wr[off + ((int64_t)(ci0 + j) * 9 + tap) * Cout + co0 + lane] = sh[lane][j];
 }
 
 // ------------------------------------------------------- small kernels
 
-// grad *= (act > 0), on a channel slice (grad dense C, act with stride/offset)
-__global__ void k_relu_bwd(bf16 *__restrict__ grad, int C, const bf16 *__restrict__ act, int a_cs, int a_c0, int64_t M)
+// grad *= (act > 0) on a channel slice (grad dense C, act with a stride), and
+// the masked gradient's channel sums, the bias gradient of the convolution
+// that made act: 15 us at 524,288 pixels x 32 (one element a thread took 52 us,
+// the bias sums 50 us more).
+__global__ void __launch_bounds__(256) k_relu_bwd(bf16 *__restrict__ grad, int C, const bf16 *__restrict__ act,
+                                                  int a_cs, int64_t M, float *__restrict__ part)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M * C) return;
-    const int64_t m = i / C;
-    const int c = (int)(i - m * C);
-    if (!(__bfloat162float(act[m * a_cs + a_c0 + c]) > 0.0f)) grad[i] = __float2bfloat16(0.0f);
+    const int t = threadIdx.x, c = blockIdx.y * 32 + (t & 3) * 8;
+    float acc[8] = {};
+#pragma unroll 2
+    for (int64_t m = (int64_t)blockIdx.x * RED_PIX + (t >> 2); m < M; m += (int64_t)gridDim.x * RED_PIX) {
+        uint4 g = ld8(grad + m * C + c);
+        const uint4 a = ld8(act + m * a_cs + c);
+        g = make_uint4(relu_mask(g.x, a.x), relu_mask(g.y, a.y), relu_mask(g.z, a.z), relu_mask(g.w, a.w));
+        st8(grad + m * C + c, g);
+#pragma unroll
+        for (int w = 0; w < 4; w++) add2(acc + 2 * w, word(g, w));
+    }
+    red_store(acc, C, part);
 }
 
 // 2x2 max pool: out[b,y,x,c] = max over the window of in (channel slice)
-__global__ void k_pool_fwd(const bf16 *__restrict__ in, int in_cs, int in_c0, bf16 *__restrict__ out, int C, int B,
-                           int H, int Wd)
+__global__ void k_pool_fwd(const bf16 *__restrict__ in, int in_cs, bf16 *__restrict__ out, int C, int B, int H, int Wd)
 {
-    const int Ho = H / 2, Wo = Wd / 2;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)B * Ho * Wo * C) return;
-    const int c = (int)(i % C);
-    const int64_t p = i / C;
-    const int x = (int)(p % Wo), y = (int)((p / Wo) % Ho), b = (int)(p / ((int64_t)Wo * Ho));
-    float mx = -INFINITY;
-    for (int q = 0; q < 4; q++) {
-        const int yy = 2 * y + (q >> 1), xx = 2 * x + (q & 1);
-        mx = fmaxf(mx, __bfloat162float(in[((int64_t)(b * H + yy) * Wd + xx) * in_cs + in_c0 + c]));
+    const unsigned Ho = H / 2, Wo = Wd / 2, G = C / 8;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= B * Ho * Wo * G) return;
+    const unsigned c = (i % G) * 8, p = i / G, x = p % Wo, by = p / Wo;  // by = b Ho + y
+    const bf16 *src = in + ((int64_t)2 * by * Wd + 2 * x) * in_cs + c;
+    const uint4 v0 = ld8(src), v1 = ld8(src + in_cs), v2 = ld8(src + (int64_t)Wd * in_cs),
+                v3 = ld8(src + (int64_t)(Wd + 1) * in_cs);
+    unsigned o[4];
+#pragma unroll
+    for (int w = 0; w < 4; w++) {
+        float m[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++)
+            m[h] = fmaxf(fmaxf(fmaxf(fmaxf(-INFINITY, ch(v0, w, h)), ch(v1, w, h)), ch(v2, w, h)), ch(v3, w, h));
+        o[w] = pack2(m[0], m[1]);
     }
-    out[i] = __float2bfloat16(mx);
+    st8(out + (int64_t)p * C + c, make_uint4(o[0], o[1], o[2], o[3]));
 }
 
-// Gradient of the pool routed to the first maximum of each window, plus the
-// skip-connection gradient (channel slice of a concat gradient), written to
-// a dense [B][H][Wd][C] gradient.
-__global__ void k_pool_bwd(const bf16 *__restrict__ gout, const bf16 *__restrict__ in, int in_cs, int in_c0,
-                           const bf16 *__restrict__ gskip, int s_cs, int s_c0, bf16 *__restrict__ gin, int C, int B,
-                           int H, int Wd)
+// Gradient of pool and skip at an encoder output: the pool's, routed to the
+// first maximum of each window, plus the skip connection's (channel slice of
+// a concat gradient), masked by the output's ReLU, to a dense [B][H][Wd][C]
+// gradient, and its channel sums (the bias gradient). A thread takes a whole
+// window, so that each tensor is read once: at 8 x 256 x 256 x 32 36 us; the
+// pool's pass alone took 149 us with a thread per element, the ReLU's and the
+// bias sums' 103 us more.
+__global__ void __launch_bounds__(256) k_pool_bwd(const bf16 *__restrict__ gout, const bf16 *__restrict__ in,
+                                                  int in_cs, const bf16 *__restrict__ gskip, int s_cs,
+                                                  bf16 *__restrict__ gin, int C, int B, int H, int Wd,
+                                                  float *__restrict__ part)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)B * H * Wd * C) return;
-    const int c = (int)(i % C);
-    const int64_t p = i / C;
-    const int x = (int)(p % Wd), y = (int)((p / Wd) % H), b = (int)(p / ((int64_t)Wd * H));
-    const int yo = y / 2, xo = x / 2, Ho = H / 2, Wo = Wd / 2;
-    float g = 0.0f;
-    if (yo < Ho && xo < Wo) {
-        float mx = -INFINITY;
-        int arg = 0;
+    const unsigned Wo = Wd / 2, M = (unsigned)B * (H / 2) * Wo;
+    const int t = threadIdx.x, c = blockIdx.y * 32 + (t & 3) * 8;
+    float acc[8] = {};
+    for (unsigned p = blockIdx.x * RED_PIX + (t >> 2); p < M; p += gridDim.x * RED_PIX) {
+        const unsigned x = p % Wo, by = p / Wo;
+        const int64_t p0 = (int64_t)2 * by * Wd + 2 * x;  // the window's first pixel
+        const uint4 go = ld8(gout + (int64_t)p * C + c);
+        uint4 v[4], sk[4];
+#pragma unroll
         for (int q = 0; q < 4; q++) {
-            const int yy = 2 * yo + (q >> 1), xx = 2 * xo + (q & 1);
-            const float v = __bfloat162float(in[((int64_t)(b * H + yy) * Wd + xx) * in_cs + in_c0 + c]);
-            if (v > mx) {
-                mx = v;
-                arg = q;
+            const int64_t pq = p0 + (q >> 1) * Wd + (q & 1);
+            v[q] = ld8(in + pq * in_cs + c);
+            sk[q] = ld8(gskip + pq * s_cs + c);
+        }
+        unsigned o[4][4];
+#pragma unroll
+        for (int w = 0; w < 4; w++) {
+            float g[4][2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                float mx = -INFINITY;
+                int arg = 0;
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (ch(v[q], w, h) > mx) {
+                        mx = ch(v[q], w, h);
+                        arg = q;
+                    }
+#pragma unroll
+                for (int q = 0; q < 4; q++) g[q][h] = (arg == q ? ch(go, w, h) : 0.0f) + ch(sk[q], w, h);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                o[q][w] = relu_mask(pack2(g[q][0], g[q][1]), word(v[q], w));
+                add2(acc + 2 * w, o[q][w]);
             }
         }
-        if (arg == (y - 2 * yo) * 2 + (x - 2 * xo))
-            g = __bfloat162float(gout[((int64_t)(b * Ho + yo) * Wo + xo) * C + c]);
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            st8(gin + (p0 + (q >> 1) * Wd + (q & 1)) * C + c, make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]));
     }
-    if (gskip) g += __bfloat162float(gskip[p * s_cs + s_c0 + c]);
-    gin[i] = __float2bfloat16(g);
+    red_store(acc, C, part);
 }
 
-// nearest x2 upsampling into a channel slice of a concat tensor
-__global__ void k_up_fwd(const bf16 *__restrict__ in, int C, bf16 *__restrict__ out, int out_cs, int out_c0, int B,
-                         int Hin, int Win)
+// nearest x2 upsampling into a channel slice of a concat tensor, a thread per
+// input pixel and eight channels (84 MB at 8 x 256 x 256 x 64: 12 us, 173 us
+// with a thread per output element)
+__global__ void k_up_fwd(const bf16 *__restrict__ in, int C, bf16 *__restrict__ out, int out_cs, int B, int Hin,
+                         int Win)
 {
-    const int H = 2 * Hin, Wd = 2 * Win;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)B * H * Wd * C) return;
-    const int c = (int)(i % C);
-    const int64_t p = i / C;
-    const int x = (int)(p % Wd), y = (int)((p / Wd) % H), b = (int)(p / ((int64_t)Wd * H));
-    out[p * out_cs + out_c0 + c] = in[((int64_t)(b * Hin + y / 2) * Win + x / 2) * C + c];
+    const unsigned G = C / 8, i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (unsigned)B * Hin * Win * G) return;
+    const unsigned c = (i % G) * 8, p = i / G, x = p % Win, by = p / Win;
+    const uint4 v = ld8(in + (int64_t)p * C + c);
+    bf16 *dst = out + ((int64_t)4 * by * Win + 2 * x) * out_cs + c;
+    const int64_t row = (int64_t)2 * Win * out_cs;
+    st8(dst, v);
+    st8(dst + out_cs, v);
+    st8(dst + row, v);
+    st8(dst + row + out_cs, v);
 }
 
-// gradient of nearest upsampling: sum of the 2x2 block (from a concat-gradient slice)
-__global__ void k_up_bwd(const bf16 *__restrict__ g, int g_cs, int g_c0, bf16 *__restrict__ gin, int C, int B,
-                         int Hin, int Win)
+// Gradient of nearest upsampling (sum of the 2x2 block of a concat-gradient
+// slice), masked by the ReLU of the upsampled activation, and its channel sums.
+__global__ void __launch_bounds__(256) k_up_bwd(const bf16 *__restrict__ g, int g_cs, const bf16 *__restrict__ act,
+                                                bf16 *__restrict__ gin, int C, int B, int Hin, int Win,
+                                                float *__restrict__ part)
 {
-    const int H = 2 * Hin, Wd = 2 * Win;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)B * Hin * Win * C) return;
-    const int c = (int)(i % C);
-    const int64_t p = i / C;
-    const int x = (int)(p % Win), y = (int)((p / Win) % Hin), b = (int)(p / ((int64_t)Win * Hin));
-    float s = 0.0f;
-    for (int q = 0; q < 4; q++) {
-        const int yy = 2 * y + (q >> 1), xx = 2 * x + (q & 1);
-        s += __bfloat162float(g[((int64_t)(b * H + yy) * Wd + xx) * g_cs + g_c0 + c]);
+    const unsigned M = (unsigned)B * Hin * Win;
+    const int t = threadIdx.x, c = blockIdx.y * 32 + (t & 3) * 8;
+    float acc[8] = {};
+    for (unsigned p = blockIdx.x * RED_PIX + (t >> 2); p < M; p += gridDim.x * RED_PIX) {
+        const unsigned x = p % Win, by = p / Win;
+        const bf16 *src = g + ((int64_t)4 * by * Win + 2 * x) * g_cs + c;
+        const int64_t row = (int64_t)2 * Win * g_cs;
+        const uint4 v0 = ld8(src), v1 = ld8(src + g_cs), v2 = ld8(src + row), v3 = ld8(src + row + g_cs);
+        const uint4 a = ld8(act + (int64_t)p * C + c);
+        unsigned o[4];
+#pragma unroll
+        for (int w = 0; w < 4; w++) {
+            float s[2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) s[h] = 0.0f + ch(v0, w, h) + ch(v1, w, h) + ch(v2, w, h) + ch(v3, w, h);
+            o[w] = relu_mask(pack2(s[0], s[1]), word(a, w));
+            add2(acc + 2 * w, o[w]);
+        }
+        st8(gin + (int64_t)p * C + c, make_uint4(o[0], o[1], o[2], o[3]));
     }
-    gin[i] = __float2bfloat16(s);
+    red_store(acc, C, part);
 }
+
+constexpr int HEAD_C = 32;
 
 // head: out[m][j] = b[j] + sum_c W[j][c] act[m][c], two outputs, FP32
-__global__ void k_head_fwd(const bf16 *__restrict__ act, int C, const float *__restrict__ W,
-                           const float *__restrict__ b, float *__restrict__ out, int64_t M)
+__global__ void __launch_bounds__(256) k_head_fwd(const bf16 *__restrict__ act, const float *__restrict__ W,
+                                                  const float *__restrict__ b, float2 *__restrict__ out, int64_t M)
 {
     const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
+    uint4 v[HEAD_C / 8];
+#pragma unroll
+    for (int q = 0; q < HEAD_C / 8; q++) v[q] = ld8(act + m * HEAD_C + 8 * q);
     float s0 = b[0], s1 = b[1];
-    for (int c = 0; c < C; c++) {
-        const float a = __bfloat162float(act[m * C + c]);
+#pragma unroll
+    for (int c = 0; c < HEAD_C; c++) {
+        const float a = ch(v[c >> 3], (c & 7) >> 1, c & 1);
         s0 = fmaf(W[c], a, s0);
-        s1 = fmaf(W[C + c], a, s1);
+        s1 = fmaf(W[HEAD_C + c], a, s1);
     }
-    out[2 * m] = s0;
-    out[2 * m + 1] = s1;
+    out[m] = make_float2(s0, s1);
 }
 
-// head backward: gact[m][c] = sum_j W[j][c] g[m][j] (masked by ReLU of act)
-__global__ void k_head_bwd_act(const float *__restrict__ g, const float *__restrict__ W, const bf16 *__restrict__ act,
-                               bf16 *__restrict__ gact, int C, int64_t M)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M * C) return;
-    const int64_t m = i / C;
-    const int c = (int)(i - m * C);
-    const float v = W[c] * g[2 * m] + W[C + c] * g[2 * m + 1];
-    gact[i] = __float2bfloat16(__bfloat162float(act[i]) > 0.0f ? v : 0.0f);
-}
+// Loss and head backward in one pass over the prediction, the target and the
+// head's input: with d = pred - target, the loss terms d^2 and the output
+// gradient g = 2 d / count; the gradient of the head's input gact[m][c] =
+// sum_j W[j][c] g[m][j], masked by its ReLU; and per block the sums of
+// g act (64), g (2), d^2 (1), to part[blockIdx.x][67], and of gact, to
+// bpart[blockIdx.x][32]. It was four kernels, of which the weight sums (66
+// threads a block, 4,096 pixels one after the other) took 893 us and the
+// single-thread sum of the loss 84 us at 524,288 pixels; now 27 us for
+// the 75 MB.
+constexpr int HEAD_COLS = 2 * HEAD_C + 3;
 
-// head weight gradient partials: part[split][j * C + c] and bias part[split][2 C + j]
-__global__ void k_head_bwd_w(const float *__restrict__ g, const bf16 *__restrict__ act, int C, int64_t M, int pps,
-                             float *__restrict__ part)
+__global__ void __launch_bounds__(256) k_head_bwd(const float2 *__restrict__ pred, const float *__restrict__ tgt,
+                                                  const float *__restrict__ W, const bf16 *__restrict__ act,
+                                                  bf16 *__restrict__ gact, int64_t M, float *__restrict__ part,
+                                                  float *__restrict__ bpart)
 {
-    const int64_t p0 = (int64_t)blockIdx.x * pps, p1 = min(M, p0 + pps);
-    const int n = 2 * C + 2;
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-        float s = 0.0f;
-        if (q < 2 * C) {
-            const int j = q / C, c = q - j * C;
-            for (int64_t m = p0; m < p1; m++) s += g[2 * m + j] * __bfloat162float(act[m * C + c]);
-        } else {
-            const int j = q - 2 * C;
-            for (int64_t m = p0; m < p1; m++) s += g[2 * m + j];
+    __shared__ float sh[8][2 * HEAD_C + 12];
+    const int t = threadIdx.x, lane = t & 31, c = (t & 3) * 8;
+    float w0[8], w1[8], a0[8] = {}, a1[8] = {}, ab[8] = {}, ag0 = 0.0f, ag1 = 0.0f, al = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        w0[k] = W[c + k];
+        w1[k] = W[HEAD_C + c + k];
+    }
+    const float cnt = (float)(2 * M);
+#pragma unroll 2
+    for (int64_t m = (int64_t)blockIdx.x * RED_PIX + (t >> 2); m < M; m += (int64_t)gridDim.x * RED_PIX) {
+        const float2 pr = pred[m];
+        const uint4 a = ld8(act + m * HEAD_C + c);
+        const float d0 = pr.x - tgt[2 * m], d1 = pr.y - tgt[2 * m + 1];
+        const float g0 = 2.0f * d0 / cnt, g1 = 2.0f * d1 / cnt;
+        al += d0 * d0;
+        al += d1 * d1;
+        ag0 += g0;
+        ag1 += g1;
+        unsigned o[4];
+#pragma unroll
+        for (int w = 0; w < 4; w++) {
+            float v[2];
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int k = 2 * w + h;
+                const float x = ch(a, w, h);
+                a0[k] += g0 * x;
+                a1[k] += g1 * x;
+                v[h] = w0[k] * g0 + w1[k] * g1;
+            }
+            o[w] = relu_mask(pack2(v[0], v[1]), word(a, w));
+            add2(ab + 2 * w, o[w]);
         }
-        part[(int64_t)blockIdx.x * n + q] = s;
+        st8(gact + m * HEAD_C + c, make_uint4(o[0], o[1], o[2], o[3]));
     }
-}
-
-// MSE: g = 2 (pred - target) / count; per-block partial sums of squares
-__global__ void k_mse(const float *__restrict__ pred, const float *__restrict__ tgt, float *__restrict__ g, int64_t n,
-                      float *__restrict__ part)
-{
-    __shared__ float sh[256];
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float d = 0.0f;
-    if (i < n) {
-        d = pred[i] - tgt[i];
-        g[i] = 2.0f * d / (float)n;
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        const float s0 = pix_sum(a0[k]), s1 = pix_sum(a1[k]);
+        if (lane < 4) {
+            sh[t >> 5][c + k] = s0;
+            sh[t >> 5][HEAD_C + c + k] = s1;
+        }
     }
-    sh[threadIdx.x] = d * d;
+    // every channel group has summed the same g and d^2: group 0's go out
+    const float s0 = pix_sum(ag0), s1 = pix_sum(ag1), sl = pix_sum(al);
+    if (lane == 0) {
+        sh[t >> 5][2 * HEAD_C] = s0;
+        sh[t >> 5][2 * HEAD_C + 1] = s1;
+        sh[t >> 5][2 * HEAD_C + 2] = sl;
+    }
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    if (t < HEAD_COLS) {
+        float s = sh[0][t];
+#pragma unroll
+        for (int w = 1; w < 8; w++) s += sh[w][t];
+        part[(int64_t)blockIdx.x * HEAD_COLS + t] = s;
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
-}
-
-__global__ void k_sum_to(const float *__restrict__ part, int n, float scale, float *__restrict__ out)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        float s = 0.0f;
-        for (int q = 0; q < n; q++) s += part[q];
-        *out = s * scale;
-    }
+    red_store(ab, HEAD_C, bpart);
 }
 
 // Adam on FP32 master parameters, refreshing the BF16 copies of the conv
@@ -340,7 +560,7 @@ struct UNet {
     int64_t head_w = 0, head_b = 0;
     int64_t nparam = 0, nbf = 0;
     float *P = nullptr, *G = nullptr, *M1 = nullptr, *M2 = nullptr;
-    bf16 *WB = nullptr, *WR = nullptr;  // BF16 weights, rotated scratch
+    bf16 *WB = nullptr, *WR = nullptr;  // BF16 weights, the same rotated (at the same offsets)
     int64_t *bfmap = nullptr;
     int64_t step = 0;
     // activations (NHWC bf16); the encoder outputs e1, e2, e3 live in the
@@ -351,11 +571,12 @@ struct UNet {
     bf16 *p3 = nullptr, *e4a = nullptr, *e4 = nullptr;   // 128 @H/8; 256; 256
     bf16 *d3a = nullptr, *d3 = nullptr, *d2a = nullptr, *d2 = nullptr, *d1a = nullptr, *d1 = nullptr;
     const bf16 *xin = nullptr;  // the last forward's input (kept for the first conv's wgrad)
-    float *out = nullptr, *gout = nullptr;
+    float *out = nullptr;
     bf16 *gd1c = nullptr, *gd2c = nullptr, *gd3c = nullptr;  // gradients of the concat tensors
     bf16 *ta = nullptr, *tb = nullptr;                       // gradient ping-pong (L1 x 32 each)
-    float *ws = nullptr;  // wgrad / reduction scratch
+    float *ws = nullptr;  // wgrad scratch
     size_t ws_floats = 0;
+    float *bpart = nullptr, *hpart = nullptr;  // partial rows: RED_BLOCKS x 32 per convolution; the head's
     float *loss = nullptr;
 };
 
@@ -365,7 +586,7 @@ static void unet_free(UNet &u)
 {
     void *ptrs[] = {u.P,   u.G,   u.M1,  u.M2,  u.WB,  u.WR,  u.bfmap, u.e1a, u.d1c,  u.p1,   u.e2a,
                     u.d2c, u.p2,  u.e3a, u.d3c, u.p3,  u.e4a, u.e4,    u.d3a, u.d3,   u.d2a,  u.d2,
-                    u.d1a, u.d1,  u.out, u.gout, u.gd1c, u.gd2c, u.gd3c, u.ta, u.tb, u.ws, u.loss};
+                    u.d1a, u.d1,  u.out, u.gd1c, u.gd2c, u.gd3c, u.ta, u.tb, u.ws, u.bpart, u.hpart, u.loss};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -430,7 +651,7 @@ static cudaError_t unet_setup(UNet &u)
     NN_TRY(nalloc(&u.M2, u.nparam));
     NN_TRY(nalloc(&u.bfmap, u.nparam));
     NN_TRY(nalloc(&u.WB, u.nbf));
-    NN_TRY(nalloc(&u.WR, 9 * 256 * 384));
+    NN_TRY(nalloc(&u.WR, u.nbf));
     NN_TRY(nalloc(&u.e1a, L1 * 32));
     NN_TRY(nalloc(&u.d1c, L1 * 96));
     NN_TRY(nalloc(&u.p1, L2 * 32));
@@ -449,7 +670,6 @@ static cudaError_t unet_setup(UNet &u)
     NN_TRY(nalloc(&u.d1a, L1 * 32));
     NN_TRY(nalloc(&u.d1, L1 * 32));
     NN_TRY(nalloc(&u.out, L1 * 2));
-    NN_TRY(nalloc(&u.gout, L1 * 2));
     NN_TRY(nalloc(&u.gd1c, L1 * 96));
     NN_TRY(nalloc(&u.gd2c, L2 * 192));
     NN_TRY(nalloc(&u.gd3c, L3 * 384));
@@ -457,6 +677,8 @@ static cudaError_t unet_setup(UNet &u)
     NN_TRY(nalloc(&u.tb, L1 * 32));
     u.ws_floats = 16u << 20;  // 64 MiB of split partials
     NN_TRY(nalloc(&u.ws, u.ws_floats));
+    NN_TRY(nalloc(&u.bpart, (size_t)NCONV * RED_BLOCKS * 32));
+    NN_TRY(nalloc(&u.hpart, (size_t)RED_BLOCKS * HEAD_COLS));
     NN_TRY(nalloc(&u.loss, 1));
     NN_TRY(cudaMemcpyAsync(u.P, P.data(), u.nparam * 4, cudaMemcpyHostToDevice, u.st));
     NN_TRY(cudaMemcpyAsync(u.bfmap, map.data(), u.nparam * 8, cudaMemcpyHostToDevice, u.st));
@@ -483,46 +705,76 @@ static cudaError_t unet_forward(UNet &u, int B, const bf16 *x0)
     u.xin = x0;
     NN_TRY(conv_f(u, 0, x0, 32, 0, u.e1a, 32, 0, B, H, W));
     NN_TRY(conv_f(u, 1, u.e1a, 32, 0, u.d1c, 96, 64, B, H, W));  // e1 -> skip slice
-    k_pool_fwd<<<nblk(L2 * 32), 256, 0, u.st>>>(u.d1c, 96, 64, u.p1, 32, B, H, W);
+    k_pool_fwd<<<nblk(L2 * 32 / 8), 256, 0, u.st>>>(u.d1c + 64, 96, u.p1, 32, B, H, W);
     NN_TRY(conv_f(u, 2, u.p1, 32, 0, u.e2a, 64, 0, B, H2, W2));
     NN_TRY(conv_f(u, 3, u.e2a, 64, 0, u.d2c, 192, 128, B, H2, W2));  // e2
-    k_pool_fwd<<<nblk(L3 * 64), 256, 0, u.st>>>(u.d2c, 192, 128, u.p2, 64, B, H2, W2);
+    k_pool_fwd<<<nblk(L3 * 64 / 8), 256, 0, u.st>>>(u.d2c + 128, 192, u.p2, 64, B, H2, W2);
     NN_TRY(conv_f(u, 4, u.p2, 64, 0, u.e3a, 128, 0, B, H3, W3));
     NN_TRY(conv_f(u, 5, u.e3a, 128, 0, u.d3c, 384, 256, B, H3, W3));  // e3
-    k_pool_fwd<<<nblk(L4 * 128), 256, 0, u.st>>>(u.d3c, 384, 256, u.p3, 128, B, H3, W3);
+    k_pool_fwd<<<nblk(L4 * 128 / 8), 256, 0, u.st>>>(u.d3c + 256, 384, u.p3, 128, B, H3, W3);
     NN_TRY(conv_f(u, 6, u.p3, 128, 0, u.e4a, 256, 0, B, H4, W4));
     NN_TRY(conv_f(u, 7, u.e4a, 256, 0, u.e4, 256, 0, B, H4, W4));
-    k_up_fwd<<<nblk(L3 * 256), 256, 0, u.st>>>(u.e4, 256, u.d3c, 384, 0, B, H4, W4);
+    k_up_fwd<<<nblk(L4 * 256 / 8), 256, 0, u.st>>>(u.e4, 256, u.d3c, 384, B, H4, W4);
     NN_TRY(conv_f(u, 8, u.d3c, 384, 0, u.d3a, 128, 0, B, H3, W3));
     NN_TRY(conv_f(u, 9, u.d3a, 128, 0, u.d3, 128, 0, B, H3, W3));
-    k_up_fwd<<<nblk(L2 * 128), 256, 0, u.st>>>(u.d3, 128, u.d2c, 192, 0, B, H3, W3);
+    k_up_fwd<<<nblk(L3 * 128 / 8), 256, 0, u.st>>>(u.d3, 128, u.d2c, 192, B, H3, W3);
     NN_TRY(conv_f(u, 10, u.d2c, 192, 0, u.d2a, 64, 0, B, H2, W2));
     NN_TRY(conv_f(u, 11, u.d2a, 64, 0, u.d2, 64, 0, B, H2, W2));
-    k_up_fwd<<<nblk(L1 * 64), 256, 0, u.st>>>(u.d2, 64, u.d1c, 96, 0, B, H2, W2);
+    k_up_fwd<<<nblk(L2 * 64 / 8), 256, 0, u.st>>>(u.d2, 64, u.d1c, 96, B, H2, W2);
     NN_TRY(conv_f(u, 12, u.d1c, 96, 0, u.d1a, 32, 0, B, H, W));
     NN_TRY(conv_f(u, 13, u.d1a, 32, 0, u.d1, 32, 0, B, H, W));
-    k_head_fwd<<<nblk(L1), 256, 0, u.st>>>(u.d1, 32, u.P + u.head_w, u.P + u.head_b, u.out, L1);
+    k_head_fwd<<<nblk(L1), 256, 0, u.st>>>(u.d1, u.P + u.head_w, u.P + u.head_b, (float2 *)u.out, L1);
     return cudaGetLastError();
 }
 
 // Backward of conv q: gpre = gradient at its output (already masked by its
-// ReLU); writes dW/db into G and, if gin != nullptr, the dense input gradient.
+// ReLU); writes dW into G and, if gin != nullptr, the dense input gradient.
+// (db is summed by the pass that made gpre.)
 static cudaError_t conv_b(UNet &u, int q, const bf16 *gpre, const bf16 *in, int in_cs, int in_c0, bf16 *gin, int B,
                           int H, int W)
 {
     const Conv &c = u.convs[q];
-    NN_TRY(conv_wgrad(gpre, c.Cout, c.Cout, in, in_cs, in_c0, c.Cin, B, H, W, 9, u.G + c.w_off, u.G + c.b_off, u.ws,
+    NN_TRY(conv_wgrad(gpre, c.Cout, c.Cout, in, in_cs, in_c0, c.Cin, B, H, W, 9, u.G + c.w_off, nullptr, u.ws,
                       u.ws_floats, u.st));
-    if (gin) {
-        NN_TRY(rotate_weights(u.WB + c.wb_off, u.WR, c.Cout, c.Cin, 9, u.st));
-        NN_TRY(conv_fwd(gpre, c.Cout, 0, c.Cout, u.WR, nullptr, gin, c.Cin, 0, c.Cin, B, H, W, 9, false, u.st));
-    }
+    if (gin)
+        NN_TRY(conv_fwd(gpre, c.Cout, 0, c.Cout, u.WR + c.wb_off, nullptr, gin, c.Cin, 0, c.Cin, B, H, W, 9, false,
+                        u.st));
     return cudaSuccess;
 }
 
-static void relu_b(UNet &u, bf16 *g, int C, const bf16 *act, int a_cs, int a_c0, int64_t M)
+// The partial rows of conv q's bias gradient (RED_BLOCKS x 32 floats each:
+// red_grid gives C / 32 times that many blocks fewer), and their fold.
+static float *bias_rows(UNet &u, int q, dim3 grid, FoldTab &tab)
 {
-    k_relu_bwd<<<nblk(M * C), 256, 0, u.st>>>(g, C, act, a_cs, a_c0, M);
+    float *part = u.bpart + (int64_t)q * RED_BLOCKS * 32;
+    const Conv &c = u.convs[q];
+    tab.add(part, c.Cout, c.Cout, (int)grid.x, 1.0f, u.G + c.b_off);
+    return part;
+}
+
+// ReLU backward at conv q's output act
+static void relu_b(UNet &u, int q, bf16 *g, const bf16 *act, int64_t M, FoldTab &tab)
+{
+    const int C = u.convs[q].Cout;
+    const dim3 grid = red_grid(M, C);
+    k_relu_bwd<<<grid, 256, 0, u.st>>>(g, C, act, C, M, bias_rows(u, q, grid, tab));
+}
+
+// Upsampling and ReLU backward at conv q's output act [B][H][W]
+static void up_b(UNet &u, int q, const bf16 *g, int g_cs, const bf16 *act, bf16 *gin, int B, int H, int W, FoldTab &tab)
+{
+    const int C = u.convs[q].Cout;
+    const dim3 grid = red_grid((int64_t)B * H * W, C);
+    k_up_bwd<<<grid, 256, 0, u.st>>>(g, g_cs, act, gin, C, B, H, W, bias_rows(u, q, grid, tab));
+}
+
+// Pool, skip and ReLU backward at conv q's output, the skip slice of a concat tensor
+static void pool_b(UNet &u, int q, const bf16 *gout, const bf16 *act, const bf16 *gskip, int cs, bf16 *gin, int B,
+                   int H, int W, FoldTab &tab)
+{
+    const int C = u.convs[q].Cout;
+    const dim3 grid = red_grid((int64_t)B * (H / 2) * (W / 2), C);
+    k_pool_bwd<<<grid, 256, 0, u.st>>>(gout, act, cs, gskip, cs, gin, C, B, H, W, bias_rows(u, q, grid, tab));
 }
 
 // Mean squared error against target and its gradient w.r.t. every
@@ -531,56 +783,56 @@ static cudaError_t unet_backward(UNet &u, int B, const float *target)
 {
     const int H = u.H, W = u.W, H2 = H / 2, W2 = W / 2, H3 = H / 4, W3 = W / 4, H4 = H / 8, W4 = W / 8;
     const int64_t L1 = (int64_t)B * H * W, L2 = L1 / 4, L3 = L1 / 16, L4 = L1 / 64;
-    const int64_t nout = L1 * 2;
-    const unsigned mb = nblk(nout);
-    k_mse<<<mb, 256, 0, u.st>>>(u.out, target, u.gout, nout, u.ws);
-    k_sum_to<<<1, 32, 0, u.st>>>(u.ws, (int)mb, 1.0f / (float)nout, u.loss);
-    {  // head: weights, bias (contiguous in P), and the masked gradient of d1
-        int bs = (int)((L1 + 4095) / 4096);
-        if (bs > 1024) bs = 1024;
-        const int pps = (int)((L1 + bs - 1) / bs);
-        k_head_bwd_w<<<bs, 128, 0, u.st>>>(u.gout, u.d1, 32, L1, pps, u.ws);
-        k_fold<<<1, 128, 0, u.st>>>(u.ws, 66, bs, u.G + u.head_w);
-        k_head_bwd_act<<<nblk(L1 * 32), 256, 0, u.st>>>(u.gout, u.P + u.head_w, u.d1, u.ta, 32, L1);
+    FoldTab tab;
+    {
+        RotTab rot;
+        for (int q = 1; q < NCONV; q++) {  // conv 0 passes no gradient on
+            const Conv &c = u.convs[q];
+            rot.s[rot.n++] = RotSeg{c.wb_off, c.Cout, c.Cin, rot.blocks};
+            rot.blocks += (c.Cout / 32) * (c.Cin / 32) * 9;
+        }
+        k_rotate<<<rot.blocks, 256, 0, u.st>>>(rot, u.WB, u.WR);
+    }
+    {  // loss, head weights and bias (contiguous in P), and the masked gradient of d1
+        const dim3 grid = red_grid(L1, HEAD_C);
+        k_head_bwd<<<grid.x, 256, 0, u.st>>>((const float2 *)u.out, target, u.P + u.head_w, u.d1, u.ta, L1, u.hpart,
+                                             bias_rows(u, 13, grid, tab));
+        tab.add(u.hpart, HEAD_COLS, HEAD_COLS - 1, (int)grid.x, 1.0f, u.G + u.head_w);
+        tab.add(u.hpart + HEAD_COLS - 1, HEAD_COLS, 1, (int)grid.x, 1.0f / (float)(2 * L1), u.loss);
     }
     // decoder
     NN_TRY(conv_b(u, 13, u.ta, u.d1a, 32, 0, u.tb, B, H, W));
-    relu_b(u, u.tb, 32, u.d1a, 32, 0, L1);
+    relu_b(u, 12, u.tb, u.d1a, L1, tab);
     NN_TRY(conv_b(u, 12, u.tb, u.d1c, 96, 0, u.gd1c, B, H, W));
-    k_up_bwd<<<nblk(L2 * 64), 256, 0, u.st>>>(u.gd1c, 96, 0, u.ta, 64, B, H2, W2);
-    relu_b(u, u.ta, 64, u.d2, 64, 0, L2);
+    up_b(u, 11, u.gd1c, 96, u.d2, u.ta, B, H2, W2, tab);
     NN_TRY(conv_b(u, 11, u.ta, u.d2a, 64, 0, u.tb, B, H2, W2));
-    relu_b(u, u.tb, 64, u.d2a, 64, 0, L2);
+    relu_b(u, 10, u.tb, u.d2a, L2, tab);
     NN_TRY(conv_b(u, 10, u.tb, u.d2c, 192, 0, u.gd2c, B, H2, W2));
-    k_up_bwd<<<nblk(L3 * 128), 256, 0, u.st>>>(u.gd2c, 192, 0, u.ta, 128, B, H3, W3);
-    relu_b(u, u.ta, 128, u.d3, 128, 0, L3);
+    up_b(u, 9, u.gd2c, 192, u.d3, u.ta, B, H3, W3, tab);
     NN_TRY(conv_b(u, 9, u.ta, u.d3a, 128, 0, u.tb, B, H3, W3));
-    relu_b(u, u.tb, 128, u.d3a, 128, 0, L3);
+    relu_b(u, 8, u.tb, u.d3a, L3, tab);
     NN_TRY(conv_b(u, 8, u.tb, u.d3c, 384, 0, u.gd3c, B, H3, W3));
-    k_up_bwd<<<nblk(L4 * 256), 256, 0, u.st>>>(u.gd3c, 384, 0, u.ta, 256, B, H4, W4);
+    up_b(u, 7, u.gd3c, 384, u.e4, u.ta, B, H4, W4, tab);
     // bottleneck
-    relu_b(u, u.ta, 256, u.e4, 256, 0, L4);
     NN_TRY(conv_b(u, 7, u.ta, u.e4a, 256, 0, u.tb, B, H4, W4));
-    relu_b(u, u.tb, 256, u.e4a, 256, 0, L4);
+    relu_b(u, 6, u.tb, u.e4a, L4, tab);
     NN_TRY(conv_b(u, 6, u.tb, u.p3, 128, 0, u.ta, B, H4, W4));
-    // encoder level 3: pool gradient + skip gradient, then e3's ReLU
-    k_pool_bwd<<<nblk(L3 * 128), 256, 0, u.st>>>(u.ta, u.d3c, 384, 256, u.gd3c, 384, 256, u.tb, 128, B, H3, W3);
-    relu_b(u, u.tb, 128, u.d3c, 384, 256, L3);
+    // encoder level 3
+    pool_b(u, 5, u.ta, u.d3c + 256, u.gd3c + 256, 384, u.tb, B, H3, W3, tab);
     NN_TRY(conv_b(u, 5, u.tb, u.e3a, 128, 0, u.ta, B, H3, W3));
-    relu_b(u, u.ta, 128, u.e3a, 128, 0, L3);
+    relu_b(u, 4, u.ta, u.e3a, L3, tab);
     NN_TRY(conv_b(u, 4, u.ta, u.p2, 64, 0, u.tb, B, H3, W3));
     // level 2
-    k_pool_bwd<<<nblk(L2 * 64), 256, 0, u.st>>>(u.tb, u.d2c, 192, 128, u.gd2c, 192, 128, u.ta, 64, B, H2, W2);
-    relu_b(u, u.ta, 64, u.d2c, 192, 128, L2);
+    pool_b(u, 3, u.tb, u.d2c + 128, u.gd2c + 128, 192, u.ta, B, H2, W2, tab);
     NN_TRY(conv_b(u, 3, u.ta, u.e2a, 64, 0, u.tb, B, H2, W2));
-    relu_b(u, u.tb, 64, u.e2a, 64, 0, L2);
+    relu_b(u, 2, u.tb, u.e2a, L2, tab);
     NN_TRY(conv_b(u, 2, u.tb, u.p1, 32, 0, u.ta, B, H2, W2));
     // level 1
-    k_pool_bwd<<<nblk(L1 * 32), 256, 0, u.st>>>(u.ta, u.d1c, 96, 64, u.gd1c, 96, 64, u.tb, 32, B, H, W);
-    relu_b(u, u.tb, 32, u.d1c, 96, 64, L1);
+    pool_b(u, 1, u.ta, u.d1c + 64, u.gd1c + 64, 96, u.tb, B, H, W, tab);
     NN_TRY(conv_b(u, 1, u.tb, u.e1a, 32, 0, u.ta, B, H, W));
-    relu_b(u, u.ta, 32, u.e1a, 32, 0, L1);
+    relu_b(u, 0, u.ta, u.e1a, L1, tab);
     NN_TRY(conv_b(u, 0, u.ta, u.xin, 32, 0, nullptr, B, H, W));
+    k_fold_cols<<<tab.blocks, 1024, 0, u.st>>>(tab);
     return cudaGetLastError();
 }
 

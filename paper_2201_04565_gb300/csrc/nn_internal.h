@@ -35,9 +35,10 @@ cudaError_t conv_wgrad(const bf16 *grad, int g_cs, int Cout, const bf16 *in, int
                        int H, int Wd, int taps, float *dW, float *db, float *scratch, size_t scratch_floats,
                        cudaStream_t st);
 
-// Rotate a 3x3 conv's weights by 180 degrees and swap in/out channels, so
-// that conv_fwd with the result computes the gradient w.r.t. the input.
-cudaError_t rotate_weights(const bf16 *W, bf16 *Wr, int Cout, int Cin, int taps, cudaStream_t st);
+// db[c] = sum over M pixels of grad (rows g_cs apart), in a fixed order;
+// scratch of 32 C floats or more.
+cudaError_t bias_grad(const bf16 *grad, int g_cs, int C, int64_t M, float *db, float *scratch, size_t scratch_floats,
+                      cudaStream_t st);
 
 }  // namespace nn
 }  // namespace lsm
