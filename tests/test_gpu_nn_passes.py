@@ -1,5 +1,6 @@
-"""The U-Net's passes between convolutions where their grids wrap: more pixels
-than one sweep of a reduction's blocks, scratch that limits the blocks."""
+"""The U-Net's passes between convolutions, and the convolution variants, where
+their grids wrap: more pixels than one sweep of a reduction's blocks, more
+patches than two CTAs per SM take at once, scratch that limits the blocks."""
 import numpy as np
 import pytest
 
@@ -41,6 +42,23 @@ def test_batch_gradient_is_the_mean_of_the_images_gradients(env, H, W):
     blocks = [(wo[q], bo[q]) for q in range(14)] + [(bo[q], bo[q] + R.CONVS[q][1]) for q in range(14)]
     for a, b in blocks + [(hw, hw + 64), (hb, hb + 2)]:
         assert np.linalg.norm(grad[a:b] - mean[a:b]) <= 2e-4 * np.linalg.norm(mean[a:b]), (a, b)
+
+
+@pytest.mark.parametrize("cout,B,H,W", [(32, 1, 8, 16), (32, 3, 250, 110), (96, 2, 160, 199)])
+def test_two_ctas_per_sm_forward(env, cout, B, H, W):
+    """32 input channels, 32-channel tiles: the halo variant with two CTAs on
+    an SM, one patch up to several per CTA, ragged patches."""
+    torch, nn = env
+    rng = np.random.default_rng(W)
+    x = R.bf16(rng.standard_normal((B, H, W, 32)))
+    Wt = R.bf16(0.2 * rng.standard_normal((cout, 9, 32)))
+    out = torch.zeros((B, H, W, cout), dtype=torch.bfloat16, device="cuda")
+    tx, tw = (torch.from_numpy(a.astype(np.float32)).to(torch.bfloat16).cuda() for a in (x, Wt))
+    nn.check(nn.lib().lsm_nn_conv_forward(nn.ptr(tx), 32, 0, 32, nn.ptr(tw), None, nn.ptr(out), cout, 0, cout, B, H, W,
+                                          9, 0, None))
+    ref = R.bf16(R.conv(x, Wt.reshape(cout, 3, 3, 32), np.zeros(cout)))
+    err = np.abs(out.float().cpu().numpy().astype(np.float64) - ref)
+    assert np.all(err <= 2 ** -7 * np.abs(ref) + 1e-6 * np.abs(ref).max())
 
 
 @pytest.mark.parametrize("C,M", [(32, 1), (32, 100000), (288, 5000), (64, 77825)])
