@@ -739,6 +739,15 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
 }
 
 // Device status -> lsm_status.
+static lsm_status status_of(BatchCtx &b, int st)
+{
+    if (st) {
+        b.err = (st & 2) ? "position outside the fixed-point range" : "non-finite position or velocity";
+        return LSM_ENONFINITE;
+    }
+    return LSM_OK;
+}
+
 static lsm_status batch_status(BatchCtx &b)
 {
     int st = 0;
@@ -748,11 +757,7 @@ static lsm_status batch_status(BatchCtx &b)
         b.err = std::string("synchronize: ") + cudaGetErrorString(e);
         return LSM_ECUDA;
     }
-    if (st) {
-        b.err = (st & 2) ? "position outside the fixed-point range" : "non-finite position or velocity";
-        return LSM_ENONFINITE;
-    }
-    return LSM_OK;
+    return status_of(b, st);
 }
 
 }  // namespace lsm
@@ -989,21 +994,25 @@ lsm_status lsm_batch_relax(lsm_batch *b, double tol, int64_t max_steps, int64_t 
         const int64_t nb = std::min(check_every, max_steps - done);
         e = cudaMemsetAsync(b->nactive, 0, sizeof(int), b->stream);
         if (e == cudaSuccess) e = lsm::batch_steps_graph(*b, nb, 0, 1, tol);
+        int dst = 0;
         if (e == cudaSuccess) e = cudaMemcpyAsync(&nact, b->nactive, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&dst, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         if (e != cudaSuccess) return bcuda(b, e, "relax");
-        st = lsm::batch_status(*b);
+        st = lsm::status_of(*b, dst);
         if (st != LSM_OK) return st;
         done += nb;
     }
     // record one sample per specimen: every specimen's final state
     e = cudaMemcpyAsync(sd1.data(), b->specs, b->S * sizeof(lsm::SpecDesc), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpy2DAsync(b->samples + b->nsamples, b->cap * sizeof(lsm::DeviceSample), b->scratch,
+                              sizeof(lsm::DeviceSample), sizeof(lsm::DeviceSample), b->S, cudaMemcpyDeviceToDevice,
+                              b->stream);
+    const long long ns = b->nsamples + 1;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_nsamp, &ns, sizeof(ns), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "relax");
-    std::vector<lsm::DeviceSample> last(b->S);
-    e = cudaMemcpyAsync(last.data(), b->scratch, b->S * sizeof(lsm::DeviceSample), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "relax");
+    if (e != cudaSuccess) return bcuda(b, e, "relax record");
     bool all = true;
     int64_t su = 0;
     for (int s = 0; s < b->S; s++) {
@@ -1013,14 +1022,7 @@ lsm_status lsm_batch_relax(lsm_batch *b, double tol, int64_t max_steps, int64_t 
         all &= conv;
         if (taken) taken[s] = ts;
         if (converged) converged[s] = conv ? 1 : 0;
-        e = cudaMemcpyAsync(b->samples + (int64_t)s * b->cap + b->nsamples, &last[s], sizeof(lsm::DeviceSample),
-                            cudaMemcpyHostToDevice, b->stream);
-        if (e != cudaSuccess) return bcuda(b, e, "relax record");
     }
-    const long long ns = b->nsamples + 1;
-    e = cudaMemcpyAsync(b->d_nsamp, &ns, sizeof(ns), cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "relax record");
     b->nsamples = ns;
     b->spring_updates += su;
     if (!all) return bfail(b, LSM_ENOTCONV, "some specimens above tolerance after max_steps");
@@ -1054,12 +1056,24 @@ static cudaError_t spec_desc(lsm_batch *b, int32_t spec, lsm::SpecDesc &sd)
 lsm_status lsm_batch_get_state(lsm_batch *b, int32_t spec, double *x, double *v)
 {
     if (!spec_ok(b, spec)) return bfail(b, LSM_EINVAL, "specimen index out of range");
-    lsm_status st = lsm::batch_status(*b);
-    if (st != LSM_OK) return st;
+    const size_t bytes = 2 * b->n[spec] * sizeof(double);
+    lsm::prefault(x, bytes);
+    lsm::prefault(v, bytes);
     lsm::SpecDesc sd;
-    cudaError_t e = spec_desc(b, spec, sd);
+    int dst = 0;
+    cudaError_t e = cudaMemcpyAsync(&dst, b->status, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = spec_desc(b, spec, sd);
     if (e != cudaSuccess) return bcuda(b, e, "get_state");
+    lsm_status st = lsm::status_of(*b, dst);
+    if (st != LSM_OK) return st;
     const int64_t np = (int64_t)b->nx[spec] * b->ny[spec], n = b->n[spec], P = b->pbase[spec];
+    if (b->pix[spec].empty()) {  // a particle in every pixel: the grid's order is the canonical one
+        if (x) e = cudaMemcpyAsync(x, b->X[sd.cur] + 2 * P, 2 * np * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess && v)
+            e = cudaMemcpyAsync(v, b->VOBS + 2 * P, 2 * np * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+        return e == cudaSuccess ? LSM_OK : bcuda(b, e, "get_state");
+    }
     std::vector<double> gx(x ? 2 * np : 0), gv(v ? 2 * np : 0);
     if (x) e = cudaMemcpyAsync(gx.data(), b->X[sd.cur] + 2 * P, 2 * np * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess && v)
@@ -1069,7 +1083,7 @@ lsm_status lsm_batch_get_state(lsm_batch *b, int32_t spec, double *x, double *v)
     const std::vector<int64_t> &pix = b->pix[spec];
     for (int c = 0; c < 2; c++)
         for (int64_t p = 0; p < n; p++) {
-            const int64_t g = pix.empty() ? p : pix[p];
+            const int64_t g = pix[p];
             if (x) x[c * n + p] = gx[c * np + g];
             if (v) v[c * n + p] = gv[c * np + g];
         }
@@ -1110,6 +1124,7 @@ lsm_status lsm_batch_broken_mask(lsm_batch *b, int32_t spec, uint8_t *out, int64
 {
     if (!spec_ok(b, spec)) return bfail(b, LSM_EINVAL, "specimen index out of range");
     if (!out || cap < b->m[spec]) return bfail(b, LSM_EINVAL, "output buffer smaller than the spring count");
+    lsm::prefault(out, b->m[spec]);
     lsm_status st = lsm::batch_status(*b);
     if (st != LSM_OK) return st;
     cudaError_t e = cudaSuccess;

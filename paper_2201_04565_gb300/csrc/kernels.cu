@@ -393,7 +393,7 @@ void free_device(Ctx &c)
     for (void *p : ptrs)
         if (p) cudaFree(p);
     void *tptrs[] = {c.tx[0], c.tx[1], c.tvh[0], c.tvh[1], c.tvobs, c.tph, c.tmask, c.tbrk, c.tmass,
-                     c.tinvm, c.tdf, c.tsbase, c.texport, c.texport_brk, c.xf, c.sdir, c.imass, c.fsx,
+                     c.tinvm, c.tdf, c.tsbase, c.texport, c.texport_brk, c.tcell, c.tstage, c.xf, c.sdir, c.imass, c.fsx,
                      c.tmask3, c.grip_list};
     for (void *p : tptrs)
         if (p) cudaFree(p);
@@ -404,6 +404,8 @@ void free_device(Ctx &c)
     c.fsx = nullptr;
     c.texport = nullptr;
     c.texport_brk = nullptr;
+    c.tcell = nullptr;
+    c.tstage = nullptr;
     c.tx[0] = c.tx[1] = c.tvh[0] = c.tvh[1] = c.tvobs = c.tmass = c.tinvm = nullptr;
     c.tdf = nullptr;
     c.tph = c.tmask = nullptr;
@@ -460,6 +462,82 @@ static ff split_ff(double v)
 {
     const float hi = (float)v;
     return ff{hi, (float)(v - (double)hi)};
+}
+
+// State readback of a grid with cells that hold no particle (void, or the
+// last site of the packing's odd rows): the device packs the particles of one
+// component and only those cross to the host, straight into the caller's
+// array. Copying whole grids and picking the particles on the host took 95 ms
+// for x and v of a 256^3 foam (35 % solid: 806 MB copied for 284 MB), 9
+// ms this way. A block packs 1,024 cells, four per thread, from the number of
+// particles before it; particles outside [p0, p1), the staging's current
+// range, are left out.
+constexpr int STATE_CELLS = 1024;
+constexpr int64_t STATE_STAGE = 4 << 20;  // staged doubles (32 MB)
+
+__global__ void __launch_bounds__(256) k_state_dense(const double *__restrict__ src, const uint8_t *__restrict__ phase,
+                                                     int64_t ncell, const int64_t *__restrict__ first, int64_t b0,
+                                                     int64_t p0, int64_t p1, double *__restrict__ out)
+{
+    __shared__ int wsum[8];
+    const int t = threadIdx.x, lane = t & 31;
+    const int64_t g = (b0 + blockIdx.x) * STATE_CELLS + 4 * t;
+    int cnt = 0;
+    bool has[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        has[k] = g + k < ncell && phase[g + k] != 0;
+        cnt += has[k];
+    }
+    int scan = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, scan, o);
+        if (lane >= o) scan += v;
+    }
+    if (lane == 31) wsum[t >> 5] = scan;
+    __syncthreads();
+    int64_t p = first[b0 + blockIdx.x] + scan - cnt;
+    for (int w = 0; w < t >> 5; w++) p += wsum[w];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        if (!has[k]) continue;
+        if (p >= p0 && p < p1) out[p - p0] = src[g + k];
+        p++;
+    }
+}
+
+cudaError_t tile_state(Ctx &c, const double *grid, double *host)
+{
+    if (c.n == c.tnp)  // a particle in every cell: the grid's order is the canonical one
+        return cudaMemcpyAsync(host, grid, (size_t)c.dim * c.n * sizeof(double), cudaMemcpyDeviceToHost, c.stream);
+    for (int d = 0; d < c.dim; d++)
+        for (int64_t p0 = 0; p0 < c.n; p0 += c.tstage_n) {
+            const int64_t p1 = std::min(c.n, p0 + c.tstage_n);
+            const int64_t b0 = c.tgidx[p0] / STATE_CELLS, b1 = c.tgidx[p1 - 1] / STATE_CELLS;
+            k_state_dense<<<(unsigned)(b1 - b0 + 1), 256, 0, c.stream>>>(grid + (int64_t)d * c.tnp, c.tph, c.tnp,
+                                                                        c.tcell, b0, p0, p1, c.tstage);
+            LSM_TRY(cudaGetLastError());
+            LSM_TRY(cudaMemcpyAsync(host + (int64_t)d * c.n + p0, c.tstage, (p1 - p0) * sizeof(double),
+                                    cudaMemcpyDeviceToHost, c.stream));
+        }
+    return cudaSuccess;
+}
+
+// tcell and the staging of tile_state (tgidx ascends: the particles' canonical
+// order is the grid's)
+static cudaError_t state_setup(Ctx &c)
+{
+    if (c.n == c.tnp || c.n == 0) return cudaSuccess;
+    const int64_t nb = (c.tnp + STATE_CELLS - 1) / STATE_CELLS;
+    std::vector<int64_t> first(nb);
+    for (int64_t b = 0; b < nb; b++)
+        first[b] = std::lower_bound(c.tgidx.begin(), c.tgidx.end(), b * STATE_CELLS) - c.tgidx.begin();
+    c.tstage_n = std::min(c.n, STATE_STAGE);
+    LSM_TRY(dalloc(&c.tcell, nb));
+    LSM_TRY(dalloc(&c.tstage, c.tstage_n));
+    LSM_TRY(cudaMemcpyAsync(c.tcell, first.data(), nb * sizeof(int64_t), cudaMemcpyHostToDevice, c.stream));
+    return cudaStreamSynchronize(c.stream);
 }
 
 // Tile path: state on the 2D pixel grid, both ping-pong buffers at the
@@ -596,9 +674,13 @@ cudaError_t upload(Ctx &c)
     c.m = h.m;
     if (c.tile && c.dim == 3) {
         LSM_TRY(upload_common(c));
-        return tile3_upload(c);
+        LSM_TRY(tile3_upload(c));
+        return state_setup(c);
     }
-    if (c.tile) return upload_tile(c);
+    if (c.tile) {
+        LSM_TRY(upload_tile(c));
+        return state_setup(c);
+    }
     const int64_t n = c.n, m = c.m, dn = (int64_t)h.dim * n;
     c.nblk_s = (m + TPB - 1) / TPB;
     c.nblk_p = (n + TPB - 1) / TPB;

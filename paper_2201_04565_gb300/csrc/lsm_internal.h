@@ -242,6 +242,10 @@ struct Ctx {
     int64_t *fpix = nullptr;              // [n] pixel of each particle
     uint8_t *texport = nullptr;           // [m] staging for canonical-order exports
     long long *texport_brk = nullptr;     // [m] staging for break steps
+    // tile paths whose grid has cells without a particle: state readback
+    int64_t *tcell = nullptr;             // particle number before each block of STATE_CELLS cells
+    double *tstage = nullptr;             // [tstage_n] staging of one component's particles
+    int64_t tstage_n = 0;
 
     // asynchronous readback (lsm_readback_async): a second stream for the
     // device-to-host copies, two device snapshots of the canonical mask with
@@ -304,6 +308,13 @@ bool net_from_desc(const lsm_net_desc &d, HostNet &out, std::string &err);
 // kernels.cu
 cudaError_t upload(Ctx &c);
 cudaError_t launch_init_accel(Ctx &c);
+// Map the pages of an output buffer before a device-to-host copy into it
+// (api.cpp): a page that the copy finds unmapped costs it 9 us, mapping it
+// here 1 us or less. The buffer's bytes keep their values.
+void prefault(void *p, size_t bytes) noexcept;
+// Tile paths: a grid array [dim][tnp] to host memory [dim][n], the particles
+// in canonical order (the copies are enqueued on the context's stream).
+cudaError_t tile_state(Ctx &c, const double *grid, double *host);
 cudaError_t launch_steps(Ctx &c, int64_t nsteps, bool record);
 cudaError_t launch_apply_strain(Ctx &c, double eps_old, double eps_new);
 cudaError_t launch_observe(Ctx &c, DeviceSample *dst);
