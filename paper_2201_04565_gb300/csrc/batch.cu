@@ -147,7 +147,7 @@ k_strip2d_batch(TileArgs base, const BatchTile *__restrict__ strips, int64_t n, 
                 const uint8_t *PH, uint8_t *MASK, long long *BRK, unsigned long long *fb, unsigned long long *nb,
                 int step)
 {
-    __shared__ TypeDF sdf[128];
+    __shared__ __align__(16) TypeDF sdf[128];
     __shared__ Coef4 scoef[8];
     __shared__ float smassf[8];
     __shared__ ff soff[4][3];

@@ -12,6 +12,8 @@
 // instructions instead of 108.8e6 and 112.1 us instead of 122.8, a 256^3 foam's
 // 830 us instead of 885 (775 on smaller blocks, tile3d.cu); what is left is
 // spread over pipes (issue 65%, ALU 56%, FP64 53%, FMA 48%) at 20 warps per SM.
+// F32 steps do the same (spring_f32_pair): 2048^2 90.5 -> 80.1 us, a 256^3
+// foam 864 -> 714 (smaller blocks included).
 #pragma once
 
 #include "dfloat.cuh"
@@ -155,6 +157,47 @@ __device__ __forceinline__ void spring_df_pair(const long long (&d)[DIM][2], con
         unpk(fq, f[c][0].hi, f[c][1].hi);
         unpk(fe, f[c][0].lo, f[c][1].lo);
     }
+}
+
+// Two F32 springs: e[c][q], the vectors minus their lattice vectors (o[c][q], oo =
+// |o|^2) in fixed point; types t = (k, r0, rc2, cor); whether they exist. Out: the
+// forces on the lower ends and the break test's outcome. The operations of
+// spring_f32_o (tile_body.cuh) and spring3 (tile3d.cu); the terms of r^2 - r0^2 are
+// added to cor in their order: y, x in 2D, x, y, z in 3D.
+template <int DIM>
+__device__ __forceinline__ void spring_f32_pair(const long long (&e)[DIM][2], const f32x2 (&o)[DIM], f32x2 oo,
+                                                const float4 &t0, const float4 &t1, const bool (&live)[2], float p24,
+                                                float p0, float (&f)[DIM][2], bool (&brk)[2])
+{
+    f32x2 x[DIM];
+#pragma unroll
+    for (int c = 0; c < DIM; c++) {
+        const f32x2 h = pk(__int2float_rn((int)(e[c][0] >> 24)), __int2float_rn((int)(e[c][1] >> 24)));
+        const f32x2 l = pk(__int2float_rn((int)(e[c][0] & 0xFFFFFFLL)), __int2float_rn((int)(e[c][1] & 0xFFFFFFLL)));
+        x[c] = fma2(h, splat(p24), mul2(l, splat(p0)));
+    }
+    const f32x2 two = splat(2.0f);
+    f32x2 num = pk(t0.w, t1.w);
+#pragma unroll
+    for (int q = 0; q < DIM; q++) {
+        const int c = DIM == 2 ? 1 - q : q;
+        num = fma2(fma2(o[c], two, x[c]), x[c], num);  // (2 o + e) e: the doubling is exact
+    }
+    const f32x2 r2 = add2(oo, num);
+    float a, b, na, nb;
+    unpk(r2, a, b);
+    unpk(num, na, nb);
+    brk[0] = live[0] && a > t0.z;
+    brk[1] = live[1] && b > t1.z;
+    const f32x2 ir = pk(rsqrt_approx(a), rsqrt_approx(b));
+    float da, db;
+    unpk(fma2(r2, ir, pk(t0.y, t1.y)), da, db);
+    const f32x2 s = pk(__fdividef(na, da), __fdividef(nb, db));  // r - r0
+    float ca, cb;
+    unpk(mul2(mul2(pk(t0.x, t1.x), s), ir), ca, cb);
+    const f32x2 k = pk(live[0] && !brk[0] ? ca : 0.0f, live[1] && !brk[1] ? cb : 0.0f);
+#pragma unroll
+    for (int c = 0; c < DIM; c++) unpk(mul2(k, add2(o[c], x[c])), f[c][0], f[c][1]);
 }
 
 }  // namespace lsm

@@ -8,10 +8,10 @@ namespace lsm {
 // One warp per strip of the image (strips numbered row-major, nsx across);
 // partial sums of a sample at index `strip`.
 template <int PREC, bool RATE, bool SAMPLE, int LAT, int MODE>
-__global__ void __launch_bounds__(32 * STRIP_WARPS, strip_min_ctas<PREC, SAMPLE>())
+__global__ void __launch_bounds__(32 * STRIP_WARPS, STRIP_CTAS)
 k_strip2d(TileArgs A, int R, int nsx)
 {
-    __shared__ TypeDF sdf[128];
+    __shared__ __align__(16) TypeDF sdf[128];
     __shared__ Coef4 scoef[8];
     __shared__ float smassf[8];
     __shared__ ff soff[4][3];  // per slot: o_x, o_y, |o|^2 (F32)
@@ -52,14 +52,15 @@ cudaError_t strip_resident(int &resident)
 }
 
 // Strips of `own` columns and R rows, one wave of `resident` warps, at least
-// rmin rows each; fills: strips of 8 rows would outnumber the resident warps.
-void strip_shape(int nx, int ny, int own, int resident, int rmin, int &R, int &nsx, int64_t &nstrips, bool &fills)
+// rmin rows each; fills: strips of 8 rows would outnumber `enough` warps.
+void strip_shape(int nx, int ny, int own, int resident, int rmin, int enough, int &R, int &nsx, int64_t &nstrips,
+                 bool &fills)
 {
     nsx = (nx + own - 1) / own;
     const int rows_target = std::max(1, resident / nsx);
     R = std::max(rmin, (ny + rows_target - 1) / rows_target);
     nstrips = (int64_t)nsx * ((ny + R - 1) / R);
-    fills = (int64_t)nsx * ((ny + 7) / 8) >= resident;
+    fills = (int64_t)nsx * ((ny + 7) / 8) >= enough;
 }
 
 template <int PREC, bool RATE, bool SAMPLE, int LAT, int MODE>
@@ -97,7 +98,9 @@ bool strip_supported(const Ctx &c)
 // *fills: whether the image is large enough for strips of 8 rows to occupy
 // the whole device (otherwise the square lattice's tile kernel, with more
 // CTAs in flight, is the faster choice: a warp's row-by-row sweep is
-// latency-bound when few run).
+// latency-bound when few run). F32 sweeps, shorter per row, take over at two
+// thirds of it: 600^2 (1,500 strips of 8 rows for 3,040 warps) 13.2 us on strips
+// and 12.2 on tiles, 700^2 (2,112) 15.4 and 17.6; DF 850^2 (3,103) 25.7 and 25.8.
 cudaError_t strip_geometry(Ctx &c, bool *fills)
 {
     int resident = 0;
@@ -106,7 +109,8 @@ cudaError_t strip_geometry(Ctx &c, bool *fills)
                           : (df ? strip_resident<LSM_PREC_DF, 0>(resident) : strip_resident<LSM_PREC_F32, 0>(resident));
     if (e != cudaSuccess) return e;
     bool f = false;
-    strip_shape(c.tgnx, c.tgny, STRIP_OWN, resident, c.tri ? 2 : 8, c.strip_R, c.strip_nsx, c.nstrips, f);
+    strip_shape(c.tgnx, c.tgny, STRIP_OWN, resident, c.tri ? 2 : 8, df ? resident : 2 * resident / 3, c.strip_R,
+                c.strip_nsx, c.nstrips, f);
     if (fills) *fills = f;
     return cudaSuccess;
 }

@@ -28,7 +28,8 @@
 // without being owned; the row below (y1) is loaded only.
 //
 // Every floating-point operation is the one the tile kernel performs, in the
-// same order (spring_df / spring_f32 / DfSum), so both kernels produce the
+// same order (spring_df / spring_f32 / DfSum; time steps take two springs at a
+// time, df_pair.cuh, with the same bits), so both kernels produce the
 // same states and a context or batch can switch between them from one step
 // to the next (the batch's sample steps stay on its tile list).
 #pragma once
@@ -153,6 +154,9 @@ __device__ __forceinline__ double strip_rate_x(const TileArgs &A, int gx, int pa
     return ad(X, ml(eps, sb(X, A.xc)));
 }
 
+// F32: the type table holds (k, r0, rc2, cor) as one 16-byte word per type.
+__device__ __forceinline__ const float4 *f32_types(const TypeDF *sdf) { return reinterpret_cast<const float4 *>(sdf); }
+
 // Force on the lower endpoint p of the spring p -> q in forward slot `slot`
 // (zero if either pixel holds no particle or the spring is broken). Returns
 // S_NONE (no spring, or broken before), S_BREAK (the break test fires in
@@ -174,7 +178,13 @@ __device__ __forceinline__ int strip_spring(const TileArgs &A, const PixFix &p, 
     const unsigned pp = p.pm & 0xffu, pq = q.pm & 0xffu;
     if (!pp || !pq || ((p.pm >> (8 + slot)) & 1u)) return S_NONE;
     const int shell = LAT == 0 ? (slot & 1) : (slot != 0);
-    t = sdf[(((int)(pp - 1) * A.nphase) + (int)(pq - 1)) * 2 + shell];
+    const int ti = (((int)(pp - 1) * A.nphase) + (int)(pq - 1)) * 2 + shell;
+    if constexpr (PREC == LSM_PREC_F32) {
+        const float4 v = f32_types(sdf)[ti];
+        t = TypeDF{{v.x, 0.0f}, {v.y, 0.0f}, {v.z, 0.0f}, {v.w, 0.0f}};
+    } else {
+        t = sdf[ti];
+    }
     bool b;
     if constexpr (PREC == LSM_PREC_DF) {
         b = spring_df<TEST, SAMPLE>(q.xf - p.xf, q.yf - p.yf, t, A, fx, fy, dx, st, big);
@@ -203,6 +213,42 @@ __device__ __forceinline__ void strip_pair(const TileArgs &A, const PixFix &p, c
     ff f[2][2];
     bool brk[2];
     spring_df_pair<2>(d, sdf[ia], sdf[ib], live, A.df_M, A.df_cmax, f, brk, big);
+    fax = f[0][0];
+    fbx = f[0][1];
+    fay = f[1][0];
+    fby = f[1][1];
+    ra = brk[0] ? S_BREAK : S_FORCE;
+    rb = brk[1] ? S_BREAK : S_FORCE;
+}
+
+// The same for F32 time steps.
+template <int LAT>
+__device__ __forceinline__ void strip_pair(const TileArgs &A, const PixFix &p, const PixFix &qa, int sa, int sha,
+                                           const PixFix &qb, int sb, int shb, const TypeDF *sdf, const ff (*soff)[3],
+                                           float &fax, float &fay, float &fbx, float &fby, int &ra, int &rb)
+{
+    const unsigned pp = p.pm & 0xffu, pa = qa.pm & 0xffu, pb = qb.pm & 0xffu;
+    const bool live[2] = {pp && pa && !((p.pm >> (8 + sa)) & 1u), pp && pb && !((p.pm >> (8 + sb)) & 1u)};
+    const int row = (int)(pp - 1) * A.nphase - 1;
+    const int ia = live[0] ? (row + (int)pa) * 2 + sha : 0, ib = live[1] ? (row + (int)pb) * 2 + shb : 0;
+    // lattice vectors: slots (+1,0), (-1,+1), (0,+1), (+1,+1); packing (+1,0), (-1/2,h), (+1/2,h)
+    auto ox = [&](int s) -> long long {
+        if (LAT == 0) return s == 1 ? -A.a_fix : (s == 2 ? 0 : A.a_fix);
+        return s == 0 ? A.a_fix : (s == 1 ? -(A.a_fix >> 1) : A.a_fix >> 1);
+    };
+    auto oy = [&](int s) -> long long { return s == 0 ? 0 : (LAT == 0 ? A.a_fix : A.h_fix); };
+    const long long e[2][2] = {{qa.xf - p.xf - ox(sa), qb.xf - p.xf - ox(sb)},
+                               {qa.yf - p.yf - oy(sa), qb.yf - p.yf - oy(sb)}};
+    // read from shared memory in every row: hoisted out of the sweep they spill
+    // (the two springs share |o|^2; the square lattice's vectors from the spacing
+    // alone: a register each for their components spills)
+    const float af = soff[0][0].hi;
+    auto cx = [&](int s) { return LAT == 0 ? (s == 1 ? -af : (s == 2 ? 0.0f : af)) : soff[s][0].hi; };
+    auto cy = [&](int s) { return LAT == 0 ? (s == 0 ? 0.0f : af) : soff[s][1].hi; };
+    const f32x2 o[2] = {pk(cx(sa), cx(sb)), pk(cy(sa), cy(sb))};
+    float f[2][2];
+    bool brk[2];
+    spring_f32_pair<2>(e, o, splat(soff[sa][2].hi), f32_types(sdf)[ia], f32_types(sdf)[ib], live, A.p24, A.p0, f, brk);
     fax = f[0][0];
     fbx = f[0][1];
     fay = f[1][0];
@@ -277,7 +323,13 @@ __device__ __forceinline__ void strip_tables(const TileArgs &A, TypeDF *sdf, Coe
 {
     const int tid = threadIdx.x;
     const int nt = 2 * A.nphase * A.nphase;
-    for (int q = tid; q < nt; q += blockDim.x) sdf[q] = A.tdf[q];
+    for (int q = tid; q < nt; q += blockDim.x) {
+        const TypeDF t = A.tdf[q];
+        if (PREC == LSM_PREC_F32)
+            reinterpret_cast<float4 *>(sdf)[q] = make_float4(t.k.hi, t.r0.hi, t.rc2.hi, t.cor.hi);
+        else
+            sdf[q] = t;
+    }
     if (tid < A.nphase) {
         scoef[tid] = A.coef[tid];
         smassf[tid] = (float)A.mass[tid];
@@ -399,6 +451,16 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
                 TypeDF t;
                 s0 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q0, 0, sdf, soff, f0x, f0y, dx, st, t, big);
                 strip_pair(A, P, q1, 1, 1, q3, 2, 1, sdf, f1x, f1y, f2x, f2y, s1, s2, big);
+            }
+        } else if constexpr (PREC == LSM_PREC_F32 && !SAMPLE && TEST) {
+            if constexpr (LAT == 0) {
+                strip_pair<LAT>(A, P, q0, 0, 0, N, 2, 0, sdf, soff, f0x, f0y, f2x, f2y, s0, s2);
+                strip_pair<LAT>(A, P, q1, 1, 1, q3, 3, 1, sdf, soff, f1x, f1y, f3x, f3y, s1, s3);
+            } else {
+                FT dx, st;
+                TypeDF t;
+                s0 = strip_spring<PREC, SAMPLE, TEST, LAT>(A, P, q0, 0, sdf, soff, f0x, f0y, dx, st, t, big);
+                strip_pair<LAT>(A, P, q1, 1, 1, q3, 2, 1, sdf, soff, f1x, f1y, f2x, f2y, s1, s2);
             }
         } else {
             FT dx, st;
@@ -576,10 +638,10 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
 
 }  // namespace
 
-// CTAs per SM the strip kernels are compiled for: 5 of 128 threads (up to
-// 102 registers) for the DF time step and every sample step, 6 (up to 85)
-// for the F32 time step; each fits its budget without spills.
-template <int PREC, bool SAMPLE>
-constexpr int strip_min_ctas() { return PREC == LSM_PREC_DF || SAMPLE ? 5 : 6; }
+// CTAs of 128 threads per SM the strip kernels are compiled for: up to 102
+// registers, without spills. (F32 time steps fit six CTAs with one spring at a
+// time, but two at a time spill there: 2048^2 90.5 us one at a time with six,
+// 85.9 two at a time with six, 80.1 with five.)
+constexpr int STRIP_CTAS = 5;
 
 }  // namespace lsm

@@ -126,7 +126,11 @@ constexpr int TILE_X = 32;
 // CTAs (64^2: 19.1 -> 11.7 us). Only sample steps write per-tile partial sums,
 // so the partials always come from 16-row tiles (half as many block reductions
 // as 8-row tiles would need).
+// F32 steps take 8 rows where 16-row tiles are fewer than three per SM, and 16
+// where there are more (300^2 8.5 -> 6.5 us, 400^2 9.6 -> 7.9 us with 8 rows;
+// 500^2 10.8 us with 16 rows, 11.9 with 8).
 constexpr int TILE_Y_SAMPLE = 16;
+constexpr int64_t F32_TILES_16 = 3 * 152;
 template <int PREC, bool SAMPLE>
 constexpr int tile_y() { return (PREC == LSM_PREC_DF || PREC == LSM_PREC_EXACT64) && !SAMPLE ? 8 : TILE_Y_SAMPLE; }
 
@@ -179,10 +183,9 @@ static TileArgs tile_args(Ctx &c)
     return A;
 }
 
-template <int PREC, int MODE, bool SAMPLE, bool RATE>
+template <int PREC, int MODE, bool SAMPLE, bool RATE, int TILE_Y = tile_y<PREC, SAMPLE>()>
 static cudaError_t launch_tile(Ctx &c, TileArgs A)
 {
-    constexpr int TILE_Y = tile_y<PREC, SAMPLE>();
     auto kern = k_tile2d<TILE_X, TILE_Y, PREC, MODE, SAMPLE, RATE>;
     const size_t smem = tile_smem_bytes<TILE_X, TILE_Y>(PREC);
     static bool configured = false;  // per template instance
@@ -209,7 +212,10 @@ template <int MODE, bool SAMPLE, bool RATE>
 static cudaError_t launch_tile_p(Ctx &c, TileArgs A)
 {
     switch (c.h.precision) {
-    case LSM_PREC_F32: return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE>(c, A);
+    case LSM_PREC_F32:
+        if constexpr (MODE == T_STEP && !SAMPLE)
+            if (c.ntiles < F32_TILES_16) return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE, 8>(c, A);
+        return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE>(c, A);
     case LSM_PREC_DF: return launch_tile<LSM_PREC_DF, MODE, SAMPLE, RATE>(c, A);
     default: return launch_tile<LSM_PREC_EXACT64, MODE, SAMPLE, RATE>(c, A);
     }

@@ -185,10 +185,10 @@ __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl,
     return true;
 }
 
-// The 18 springs of a particle, DF: forces into F (split sums), new breaks of its
+// The 18 springs of a particle: forces into F (split sums), new breaks of its
 // forward springs into newb; slot s's incoming spring is broken by its source's
 // flags or its own break test, which the source's thread records.
-template <typename SUM, bool TEST>
+template <int PREC, typename SUM, bool TEST>
 __device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, const TypeDF *sdf, const int *soff,
                                             int ep, int pp, uint16_t mk, const long long (&xp)[3], DfSumCareful (&F)[3],
                                             uint16_t &newb, bool &big)
@@ -212,7 +212,26 @@ __device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, 
         }
         ff f[3][2];
         bool brk[2];
-        spring_df_pair<3>(d, ti, to, live, A.df_M, A.df_cmax, f, brk, big);
+        if constexpr (PREC == LSM_PREC_DF) {
+            spring_df_pair<3>(d, ti, to, live, A.df_M, A.df_cmax, f, brk, big);
+        } else {
+            f32x2 o3[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const int k = A.sd[s][c];
+                d[c][0] -= (long long)k * A.a_fix;
+                d[c][1] -= (long long)k * A.a_fix;
+                o3[c] = splat(k == 0 ? 0.0f : (k > 0 ? A.fa : -A.fa));
+            }
+            float ff3[3][2];
+            spring_f32_pair<3>(d, o3, splat(A.oo2[sh]), make_float4(ti.k.hi, ti.r0.hi, ti.rc2.hi, ti.cor.hi),
+                               make_float4(to.k.hi, to.r0.hi, to.rc2.hi, to.cor.hi), live, A.p24, A.p0, ff3, brk);
+#pragma unroll
+            for (int c = 0; c < 3; c++) {  // in the form of a split force
+                f[c][0] = ff{-ff3[c][0], 0.0f};
+                f[c][1] = ff{-ff3[c][1], 0.0f};
+            }
+        }
         if (TEST && brk[1]) newb |= (uint16_t)(1u << s);
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -334,20 +353,21 @@ k_tile3d(Tile3Args A)
                 vpre[c] = A.vh_in[c * A.nv + g];
             }
         }
-        // one spring at a time (sample steps, and F32, whose forces are plain
-        // floats: hi alone) the sums keep their errors
+        // one spring at a time (sample steps), and in F32, whose forces are
+        // plain floats (hi alone), the sums keep their errors
         DfSumCareful F3[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) F3[c].hs = F3[c].el = 0.0f;
         uint16_t newb = 0;
-        if constexpr (PREC == LSM_PREC_DF && !SAMPLE) {
+        if constexpr (!SAMPLE) {
             // a slot's incoming (source p - o_s) and outgoing (target p + o_s)
             // springs side by side on packed instructions
             bool big = false;
-            tile3_pairs<DfSum, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
-            if (big) {  // a force beyond the split's exact range: the sums again, with their errors
+            using SUM = typename std::conditional<PREC == LSM_PREC_DF, DfSum, DfSumCareful>::type;
+            tile3_pairs<PREC, SUM, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
+            if (PREC == LSM_PREC_DF && big) {  // a force beyond the split's exact range: the sums again, with their errors
                 newb = 0;
-                tile3_pairs<DfSumCareful, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
+                tile3_pairs<PREC, DfSumCareful, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb, big);
             }
         } else {
             // incoming by ascending source (descending slot), then outgoing
