@@ -4,7 +4,8 @@
 //
 // A CTA (256 threads) owns a 16 x 8 x 8 block of voxels. Per time step it
 //   1. loads the block plus a one-voxel halo (phase, broken flags, positions
-//      drifted by dt vh, Eq. 3) into shared memory as 64-bit fixed point;
+//      drifted by dt vh, Eq. 3) into shared memory as 64-bit fixed point, and
+//      writes the block's own drifted positions, x(t+dt);
 //   2. compacts the block's particles into a list in raster order (porous
 //      volumes leave most voxels void; the list keeps every warp busy);
 //   3. for each listed particle evaluates all 18 of its springs, incoming springs by
@@ -17,7 +18,7 @@
 //      barrier per step: in 3D that exchange (9 slots x 3 components per
 //      source voxel) would cost more shared memory than the recomputation
 //      costs arithmetic in these modes;
-//      and integrates (Eqs. 4-5) in FP64, writing x(t+dt), vh(t+3dt/2).
+//      and integrates (Eqs. 4-5) in FP64, writing vh(t+3dt/2).
 // The FP64 modes keep the spring-list kernels for 3D: recomputing every
 // spring twice would double their FP64-pipe work.
 //
@@ -39,7 +40,12 @@ namespace {
 // one CTA's region load runs beside the others' springs. Against 32 x 8 x 8 blocks
 // in two CTAs of 512 the halo is a little dearer (1.76 region voxels per voxel,
 // 1.66) and the 256^3 foam's step 830 -> 775 us; 32 x 8 x 4 in three of 256: 816;
-// 16 x 8 x 4 in six of 128: 794.
+// 16 x 8 x 4 in six of 128: 794. Writing the drifted positions as they are loaded
+// (the integration no longer reads x and vh's drift again) and one warp scanning
+// the row counts take it to 754. Without the springs it takes 400: region loads
+// cost as much as arithmetic. Listing the region's particles first and loading
+// only those, two at a time, has the same instructions and more barriers (831);
+// two voxels' state in flight per thread spills (768).
 constexpr int T3X = 16, T3Y = 8, T3Z = 8, T3V = T3X * T3Y * T3Z;  // voxels per block
 constexpr int T3N = 256;                                           // threads per CTA
 constexpr int T3MIN = 4;                                           // CTAs per SM
@@ -96,6 +102,13 @@ __device__ __forceinline__ double rate_grip_x(const Tile3Args &A, int gx)
     return __dadd_rn(X, __dmul_rn(eps, __dsub_rn(X, A.xc)));
 }
 
+// Whether region voxel e belongs to the block itself (not to its halo).
+__device__ __forceinline__ bool in_block(int e)
+{
+    const int rx = e % R3X, ry = (e / R3X) % R3Y, rz = e / (R3X * R3Y);
+    return rx >= 1 && rx <= T3X && ry >= 1 && ry <= T3Y && rz >= 1 && rz <= T3Z;
+}
+
 // A region voxel on its way from memory to shared memory (g < 0: outside).
 struct RawVoxel {
     int64_t g;
@@ -113,10 +126,11 @@ __device__ __forceinline__ RawVoxel voxel_at(const Tile3Args &A, int x0, int y0,
     return r;
 }
 
-// rate_l, rate_r: the grips' x under the constant strain rate (RATE)
-template <int MODE, bool RATE>
+// rate_l, rate_r: the grips' x under the constant strain rate (RATE); own: a
+// voxel of the block itself, whose drifted position is the step's output
+template <int MODE, bool SAMPLE, bool RATE>
 __device__ __forceinline__ void load_voxel(const Tile3Args &A, int x0, int e, const RawVoxel &r, Smem3 &S, bool &over,
-                                           double rate_l, double rate_r)
+                                           bool &bad, double rate_l, double rate_r)
 {
     uint16_t mk = 0;
     double px[3] = {0.0, 0.0, 0.0};
@@ -131,6 +145,13 @@ __device__ __forceinline__ void load_voxel(const Tile3Args &A, int x0, int e, co
             if (MODE == T_STEP && !fixed) px[c] = fma(A.dt, A.vh_in[c * A.nv + r.g], px[c]);
         }
         if (RATE && MODE == T_STEP && grip) px[0] = gx == 0 ? rate_l : rate_r;
+        if (MODE == T_STEP && in_block(e)) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                A.x_out[c * A.nv + r.g] = px[c];
+                if (SAMPLE && !(grip && (c == 0 || A.grip_mode == 1))) bad |= !dbl_finite_bits(px[c]);
+            }
+        }
 #pragma unroll
         for (int c = 0; c < 3; c++) S.xf[c][e] = dbl_to_fix(px[c], A.S, over);
     }
@@ -275,7 +296,7 @@ k_tile3d(Tile3Args A)
     const long long step_now = MODE == T_STEP ? *A.d_step + A.t_off : 0;
 
     // 1. region (block + one-voxel halo) into shared memory
-    bool over = false;
+    bool over = false, bad = false;
     double rate_l = 0.0, rate_r = 0.0;  // grips' x under the constant strain rate
     if constexpr (RATE && MODE == T_STEP) {
         rate_l = rate_grip_x(A, 0);
@@ -293,7 +314,7 @@ k_tile3d(Tile3Args A)
 #pragma unroll
     for (int k = 0; k < KL; k++) {
         const int e = tid + k * T3N;
-        if (e < R3N) load_voxel<MODE, RATE>(A, x0, e, raw[k], S, over, rate_l, rate_r);
+        if (e < R3N) load_voxel<MODE, SAMPLE, RATE>(A, x0, e, raw[k], S, over, bad, rate_l, rate_r);
     }
     if (over) atomicOr(A.status, 2);
     __syncthreads();
@@ -308,14 +329,17 @@ k_tile3d(Tile3Args A)
         if (lane == 0) wcount[r] = __popc(b);
     }
     __syncthreads();
-    if (tid == 0) {
-        int acc = 0;
-        for (int r = 0; r < T3V / 32; r++) {
-            const int cnt = wcount[r];
-            wcount[r] = acc;
-            acc += cnt;
+    static_assert(T3V / 32 == 32, "one scan of 32 rows");
+    if (tid < 32) {
+        const int cnt = wcount[lane];
+        int sum = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += u;
         }
-        ntotal = acc;
+        wcount[lane] = sum - cnt;
+        if (lane == 31) ntotal = sum;
     }
     __syncthreads();
     for (int r = tid >> 5; r < T3V / 32; r += T3N / 32) {
@@ -331,7 +355,6 @@ k_tile3d(Tile3Args A)
     ff w_acc{0.0f, 0.0f}, u_acc{0.0f, 0.0f};
     float mvx2f = 0.0f, kef = 0.0f, resf = 0.0f;
     ff reactf{0.0f, 0.0f};
-    bool bad = false;
     const int count = ntotal;
     for (int i = tid; i < count; i += T3N) {
         const int ep = S.list[i];
@@ -345,13 +368,10 @@ k_tile3d(Tile3Args A)
         // here, so their latency hides behind the springs (the sample
         // instance keeps them late: it has no registers to spare)
         constexpr bool PRE = MODE == T_STEP && !SAMPLE;
-        double xpre[3], vpre[3];
+        double vpre[3];
         if constexpr (PRE) {
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                xpre[c] = A.x_in[c * A.nv + g];
-                vpre[c] = A.vh_in[c * A.nv + g];
-            }
+            for (int c = 0; c < 3; c++) vpre[c] = A.vh_in[c * A.nv + g];
         }
         // one spring at a time (sample steps), and in F32, whose forces are
         // plain floats (hi alone), the sums keep their errors
@@ -409,8 +429,7 @@ k_tile3d(Tile3Args A)
         }
         if (MODE == T_STEP && newb) A.mask[g] = (uint16_t)(mk | newb);
 
-        // integration (Eqs. 4-5), FP64; the drift is recomputed exactly as in
-        // the region load (same operations on the same inputs)
+        // integration (Eqs. 4-5), FP64
         const bool grip = gx == 0 || gx == A.nx - 1;
         const int ph = pp - 1;
         if (SAMPLE && gx == A.nx - 1) reactf = ff_add_sloppy(reactf, ff{-F3[0].hs, -F3[0].el});
@@ -421,18 +440,9 @@ k_tile3d(Tile3Args A)
             const double F = F3[c].value(A.df_bias);
             float Ff = __fadd_rn(F3[c].hs, F3[c].el);
             if (PREC == LSM_PREC_DF) Ff = __fmul_rn(Ff, A.p24);  // back from units of 2^(24-S)
-            double xr;
             double vh;
-            if constexpr (PRE) {
-                xr = xpre[c];
-                vh = vpre[c];
-            } else {
-                xr = A.x_in[q];
-                vh = MODE == T_INIT ? A.v_obs[q] : A.vh_in[q];
-            }
-            if (MODE == T_STEP && !fixed) xr = fma(A.dt, vh, xr);
-            if (RATE && MODE == T_STEP && c == 0 && grip) xr = gx == 0 ? rate_l : rate_r;
-            if (MODE == T_STEP) A.x_out[q] = xr;
+            if constexpr (PRE) vh = vpre[c];
+            else vh = MODE == T_INIT ? A.v_obs[q] : A.vh_in[q];
             if (fixed) {
                 if (MODE == T_STEP) A.vh_out[q] = 0.0;
                 if (MODE == T_STEP && SAMPLE) A.v_obs[q] = 0.0;
@@ -460,7 +470,7 @@ k_tile3d(Tile3Args A)
                 resf = fmaxf(resf, fmaxf(fabsf(Ff), fabsf(vf)));
                 kef = fmaf(0.5f * smassf[ph] * vf, vf, kef);
                 if (c == 0) mvx2f = fmaf(smassf[ph] * vf, vf, mvx2f);
-                bad |= !dbl_finite_bits(vn) || !dbl_finite_bits(xr);
+                bad |= !dbl_finite_bits(vn);
             }
         }
     }
