@@ -57,9 +57,9 @@ struct BatchCtx {
     std::vector<std::vector<int64_t>> pix;  // particle -> pixel (empty: identity)
     std::vector<double> eps;                // host mirror
     int64_t NP = 0;                         // pixels in all specimens
-    // schedule: tiles of tile_y rows, or (strip_r > 0, fixed-point modes)
-    // the plain steps on strips of strip_r rows
-    int tile_y = 16, grid = 0, order = 0, strip_r = 0;
+    // schedule: tiles of tile_y rows, or (strip_s > 0: 8, 16, 32; fixed-point
+    // modes) the time steps on strips, of strip_r rows
+    int tile_y = 16, grid = 0, order = 0, strip_s = 0, strip_r = 0;
     int64_t T = 0;
     BatchTile *strips = nullptr;  // (spec, sx, sy) of every strip
     int64_t NSTRIP = 0;
@@ -369,16 +369,53 @@ static ff split_ff_b(double v)
     return ff{hi, (float)(v - (double)hi)};
 }
 
+// Warps of the batched strip kernel that fit on the device at once (0: unknown).
+static int64_t batch_strip_slots()
+{
+    int dev = 0, nsm = 0, nb = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_strip2d_batch<LSM_PREC_DF, false>, 32 * STRIP_WARPS, 0) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return (int64_t)nb * STRIP_WARPS * nsm;
+}
+
+static int64_t batch_strips(const BatchCtx &b, int R)
+{
+    int64_t n = 0;
+    for (int s = 0; s < b.S; s++)
+        n += (int64_t)((b.nx[s] + STRIP_OWN - 1) / STRIP_OWN) * ((b.ny[s] + R - 1) / R);
+    return n;
+}
+
+// Rows per strip of the 16-row schedule: 16, or, where strips of 16 rows take
+// more than one wave of the resident warps and strips of up to 64 rows only
+// one, the least rows for one wave: a second wave that is partly empty costs
+// more than the longer sweeps (20 specimens of sides 32 to 512, 4,490 strips
+// of 16 rows for 3,040 warps: DF 77.5 us a step with
+// 16 rows, 71.4 in one wave; F32 57.6 and 50.7).
+static int batch_strip_rows(const BatchCtx &b)
+{
+    const int64_t slots = batch_strip_slots();
+    if (slots == 0 || batch_strips(b, 16) <= slots || batch_strips(b, 64) > slots) return 16;
+    int R = 17;
+    while (batch_strips(b, R) > slots) R++;
+    return R;
+}
+
 // (Re)build the tile list for tile height ty and order (0 natural, 1 largest
 // specimen first), the 16-row list of the sample steps (the same list when ty
 // is 16: the per-tile sample reductions would double on 8-row tiles) and the
 // per-tile partial buffers, which only sample steps write. ty = -R (R 8, 16
-// or 32): the plain steps run on strips of 30 owned columns and R rows, in
-// the same specimen order, and the tiles (load increments, sample steps,
+// or 32): the time steps run on strips of 30 owned columns and R rows (16:
+// batch_strip_rows), in the same specimen order, and the tiles (load increments, sample steps,
 // fields) are 16 rows high.
 static cudaError_t build_tiles(BatchCtx &b, int ty, int order)
 {
-    const int strip_r = ty < 0 ? -ty : 0;
+    const int strip_s = ty < 0 ? -ty : 0, strip_r = strip_s == 16 ? batch_strip_rows(b) : strip_s;
     if (strip_r) ty = 16;
     constexpr int TYS = 16;
     std::vector<int> sorder(b.S);
@@ -436,6 +473,7 @@ static cudaError_t build_tiles(BatchCtx &b, int ty, int order)
     BT_TRY(cudaMemcpyAsync(b.specs, sd.data(), b.S * sizeof(SpecDesc), cudaMemcpyHostToDevice, b.stream));
     BT_TRY(cudaStreamSynchronize(b.stream));
     b.tile_y = ty;
+    b.strip_s = strip_s;
     b.strip_r = strip_r;
     b.order = order;
     drop_graphs(b);
@@ -477,24 +515,6 @@ static TileArgs batch_base_args(BatchCtx &b)
     A.part_p = b.part_p;
     A.ntiles = b.TS;  // partial sums come from the sample-step tiles or strips
     return A;
-}
-
-// Whether strips of R rows outnumber the warps of the batched strip kernel
-// that fit on the device at once.
-static bool batch_strips_fill(const BatchCtx &b, int R)
-{
-    int dev = 0, nsm = 0, nb = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_strip2d_batch<LSM_PREC_DF, false>, 32 * STRIP_WARPS, 0) !=
-            cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    int64_t strips = 0;
-    for (int s = 0; s < b.S; s++)
-        strips += (int64_t)((b.nx[s] + STRIP_OWN - 1) / STRIP_OWN) * ((b.ny[s] + R - 1) / R);
-    return strips >= (int64_t)nb * STRIP_WARPS * nsm;
 }
 
 template <int PREC, bool SAMPLE>
@@ -723,12 +743,23 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     BT_TRY(cudaMemcpyAsync(b.tmass, mtab.data(), b.nphase * sizeof(double), cudaMemcpyHostToDevice, st));
     BT_TRY(cudaMemcpyAsync(b.tcoef, coef.data(), 4 * b.nphase * sizeof(double), cudaMemcpyHostToDevice, st));
     BT_TRY(cudaStreamSynchronize(st));
-    // default schedule: largest specimens first, plain steps on 16-row
-    // strips in the fixed-point modes when the strips fill the device (what
-    // the autotuner picks on the benchmark's batches; a warp sweeping a strip
-    // is latency-bound when few run), 8-row tiles otherwise (12 specimens of
-    // 128^2, a step: exact 37.4 -> 35.4 us against 16 rows, df64 11.3 -> 10.7)
-    BT_TRY(build_tiles(b, batch_strips_ok(b) && batch_strips_fill(b, 16) ? -16 : 8, 1));
+    // default schedule: largest specimens first; time steps on 16-row strips
+    // in the fixed-point modes when the strips fill the device (what the
+    // autotuner picks on the benchmark's batches; a warp sweeping a strip is
+    // latency-bound when few run), 8-row tiles otherwise (12 specimens of
+    // 128^2, a step: exact 37.4 -> 35.4 us against 16 rows, df64 11.3 -> 10.7,
+    // f32 12.3 -> 10.1). F32 sweeps pay from two thirds of the warps on, as
+    // in the single-specimen kernel, then on 8-row strips (12 specimens of
+    // sides 32 to 512: 38.2 us on tiles, 29.7 on strips).
+    const int64_t slots = batch_strips_ok(b) ? batch_strip_slots() : 0;
+    int ty = 8;
+    if (slots > 0 && b.prec == LSM_PREC_F32) {
+        const int64_t n8 = batch_strips(b, 8);
+        if (3 * n8 >= 2 * slots) ty = n8 <= slots ? -8 : -16;
+    } else if (slots > 0 && batch_strips(b, 16) >= slots) {
+        ty = -16;
+    }
+    BT_TRY(build_tiles(b, ty, 1));
     // initial acceleration of every specimen (vh = v + dt/2 a(0))
     {
         cudaError_t ei = launch_b<T_INIT, false>(b, 0, b.T);
@@ -923,7 +954,7 @@ lsm_status lsm_batch_set_schedule(lsm_batch *b, int32_t tile_y, int32_t grid, in
         return bfail(b, LSM_EINVAL, "strip schedules need the F32 or DF mode and specimens below 2^29 pixels");
     if (grid != b->grid) lsm::drop_graphs(*b);
     b->grid = grid;
-    const int cur = b->strip_r ? -b->strip_r : b->tile_y;
+    const int cur = b->strip_s ? -b->strip_s : b->tile_y;
     if (tile_y != cur || order != b->order) {
         cudaError_t e = lsm::build_tiles(*b, tile_y, order);
         if (e != cudaSuccess) return bcuda(b, e, "schedule");
@@ -1220,7 +1251,7 @@ lsm_status lsm_batch_autotune(lsm_batch *b, int32_t steps_per_trial, int32_t *ti
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     const int64_t launches0 = b->launches;
     double best = 1e300;
-    const int cur_ty = b->strip_r ? -b->strip_r : b->tile_y;
+    const int cur_ty = b->strip_s ? -b->strip_s : b->tile_y;
     int bty = cur_ty, bgrid = b->grid, bord = b->order;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (e == cudaSuccess) e = cudaEventCreate(&e0);

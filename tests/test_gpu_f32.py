@@ -62,3 +62,26 @@ def test_foam_pairs_agree_with_the_sample_step(L, shape, rate):
         g.close()
     assert np.array_equal(outs[0][2], outs[1][2])
     assert np.abs(outs[0][0] - outs[1][0]).max() <= 1e-10 and np.abs(outs[0][1] - outs[1][1]).max() <= 1e-10
+
+
+@pytest.mark.parametrize("precision,count", [("df64", 11), ("f32", 11), ("f32", 6), ("df64", 6)])
+def test_batch_strips_of_one_wave_agree_bitwise(L, precision, count):
+    """Eleven specimens near 400 x 330 take strips of more than 16 rows, so that
+    all run at once, six (F32) strips of 8: the states are those of the tiles."""
+    from paper_2201_04565_gb300 import batch as B
+    k, e, _ = two_phase_materials()
+    imgs = [inclusion_image(400 + 7 * q, 330 - 3 * q, 3.0, 9.0, 0.3, q) for q in range(count)]
+    imgs[1][100:140, 50:90] = 0
+    outs = []
+    for sched in (None, (-16, 0, 1), (8, 0, 1)):
+        b = B.Batch(imgs, k, e, precision=precision)
+        if sched:
+            b.set_schedule(*sched)
+        for i in range(1, 4):
+            b.apply_strain(0.01 * i)
+            b.step(6)
+        outs.append([(*b.state(q), b.broken(q)[0]) for q in range(count)])
+        b.close()
+    for o in outs[1:]:
+        for p, q in zip(outs[0], o):
+            assert all(np.array_equal(a, c) for a, c in zip(p, q))
