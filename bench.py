@@ -130,10 +130,10 @@ NCU_INSTRUCTIONS = {
 # Binding unit of each mode's time-step kernel, from ncu on the same workload
 # (see the profile summaries), for the roofline's "limiter" note.
 LIMITER = {
-    "df64": "instruction issue (ncu: 74% of issue slots busy, FP64 pipe 48%, DRAM 24% of peak)",
-    "f32": "instruction issue (ncu: 72% of issue slots busy, FP64 pipe 52%, DRAM 33% of peak)",
-    "fast64": "FP64 pipe (ncu: 86% busy)",
-    "exact64": "FP64 pipe (ncu: 88% busy; correctly rounded sqrt and divide)",
+    "df64": "issue and FP64 pipe (ncu: 66% of issue slots busy, ALU 56%, FP64 pipe 53%, DRAM 30% of peak)",
+    "f32": "issue and FP64 pipe",
+    "fast64": "FP64 pipe (ncu: 69% busy; the exact64 kernel)",
+    "exact64": "FP64 pipe (ncu: 69% busy; correctly rounded sqrt and divide on the integer and FP32 pipes)",
 }
 
 # Time-step kernel of each mode on the 2D image lattice.
@@ -148,10 +148,11 @@ KERNEL = {
 def _kernel_tag():
     """sha1 prefix of the 2D time-step kernels' sources (the strip kernel of
     the fixed-point modes and its sweep, the tile kernel of the FP64 modes,
-    and the arithmetic they share)."""
+    and the arithmetic they use)."""
     import hashlib
     h = hashlib.sha1()
-    for name in ("strip2d.cu", "strip_body.cuh", "tile2d.cu", "tile_body.cuh", "dfloat.cuh"):
+    for name in ("strip2d.cu", "strip_body.cuh", "tile2d.cu", "tile_body.cuh", "dfloat.cuh", "df_pair.cuh",
+                 "exact64.cuh"):
         with open(os.path.join(ROOT, "paper_2201_04565_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:12]

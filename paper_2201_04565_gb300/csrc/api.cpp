@@ -24,8 +24,12 @@ namespace lsm {
 void prefault(void *p, size_t bytes) noexcept
 {
     cudaPointerAttributes at;
-    if (!p || !bytes || cudaPointerGetAttributes(&at, p) != cudaSuccess || at.type != cudaMemoryTypeUnregistered)
-        return;  // page-locked or device memory
+    if (!p || !bytes) return;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    if (at.type != cudaMemoryTypeUnregistered) return;  // page-locked or device memory
 #ifdef MADV_POPULATE_WRITE
     // Not by touching: a read, or an atomic, maps the shared zero page first,
     // and the write fault that replaces it costs an invalidation of the GPU's
