@@ -109,10 +109,10 @@ def algorithmic_bytes(n, m, dim):
 NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum on three
     # time-step launches of each mode (the same 2048 x 2048 workload), mean
-    "df64": (238.3e6, "5ebefc3dec19"),
-    "f32": (240.1e6, "5ebefc3dec19"),
-    "fast64": (236.2e6, "5ebefc3dec19"),
-    "exact64": (236.9e6, "5ebefc3dec19"),
+    "df64": (238.5e6, "b85ff6edce8d"),
+    "f32": (238.4e6, "b85ff6edce8d"),
+    "fast64": (238.2e6, "b85ff6edce8d"),
+    "exact64": (238.0e6, "b85ff6edce8d"),
 }
 
 # Warp instructions executed by one time-step launch (ncu smsp__inst_executed.sum,
@@ -121,19 +121,19 @@ NCU_TRAFFIC = {
 # this gives the instruction-issue roofline, the one the fixed-point modes
 # are bound by.
 NCU_INSTRUCTIONS = {
-    "df64": (108821973, "5ebefc3dec19"),
-    "f32": (75982754, "5ebefc3dec19"),
-    "fast64": (94464248, "5ebefc3dec19"),
-    "exact64": (195572908, "5ebefc3dec19"),
+    "df64": (89419340, "b85ff6edce8d"),
+    "f32": (65048772, "b85ff6edce8d"),
+    "fast64": (314600626, "b85ff6edce8d"),
+    "exact64": (314600626, "b85ff6edce8d"),
 }
 
 # Binding unit of each mode's time-step kernel, from ncu on the same workload
 # (see the profile summaries), for the roofline's "limiter" note.
 LIMITER = {
     "df64": "issue and FP64 pipe (ncu: 66% of issue slots busy, ALU 56%, FP64 pipe 53%, DRAM 30% of peak)",
-    "f32": "issue and FP64 pipe",
-    "fast64": "FP64 pipe (ncu: 69% busy; the exact64 kernel)",
-    "exact64": "FP64 pipe (ncu: 69% busy; correctly rounded sqrt and divide on the integer and FP32 pipes)",
+    "f32": "issue and FP64 pipe (ncu: 67% of issue slots busy, FP64 pipe 57%, DRAM 43% of peak)",
+    "fast64": "FP64 pipe (ncu: 70% busy; the exact64 kernel)",
+    "exact64": "FP64 pipe (ncu: 70% busy; correctly rounded sqrt and divide on the integer and FP32 pipes)",
 }
 
 # Time-step kernel of each mode on the 2D image lattice.
