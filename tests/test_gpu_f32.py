@@ -85,3 +85,23 @@ def test_batch_strips_of_one_wave_agree_bitwise(L, precision, count):
     for o in outs[1:]:
         for p, q in zip(outs[0], o):
             assert all(np.array_equal(a, c) for a, c in zip(p, q))
+
+
+@pytest.mark.parametrize("eps", [-0.02, -0.15, -0.4])
+def test_df64_foam_with_large_forces_agrees_with_the_sample_step(L, eps):
+    """Double-float foams below, around and far above the split sums' exact
+    range (compressed springs have no largest force): steps without a sample
+    against steps of one, which all sample and sum with error terms. Both keep
+    a force to about 2^-44; twelve steps of dt = 0.01 leave less than 1e-12."""
+    k, e, m = two_phase_materials()
+    img = np.random.default_rng(7).integers(0, 3, size=(12, 19, 35)).astype(np.uint8)
+    outs = []
+    for calls in ((12,), (1,) * 12):
+        g = L.Specimen.from_image(img, k, e, m, precision="df64", dt=0.01)
+        g.apply_strain(eps)
+        for n in calls:
+            g.step(n)
+        outs.append((*g.state(), g.broken()[0]))
+        g.close()
+    assert np.array_equal(outs[0][2], outs[1][2])
+    assert np.abs(outs[0][0] - outs[1][0]).max() <= 1e-11 and np.abs(outs[0][1] - outs[1][1]).max() <= 1e-10
