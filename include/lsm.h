@@ -66,8 +66,10 @@ typedef enum {
  *      positions and velocities integrated in double.
  *  LSM_PREC_DF: as LSM_PREC_F32, but the spring force and the gather use
  *      double-float arithmetic (pairs of floats, 48 significant bits; 1/r by
- *      one double-float Newton step, about 2^-45), so forces carry about
- *      3e-14 relative error while the FP64 pipe only does the integration.
+ *      one double-float Newton step, about 2^-45), so the force on a particle
+ *      is off by about 3e-14 k r0 of its own springs (root mean square),
+ *      however much stiffer or stronger the other phases are, while the FP64
+ *      pipe only does the integration.
  *      In both fixed-point modes every spring vector up to the longest
  *      critical length converts exactly, and a non-finite force (which only
  *      positions already out of range can produce) is reported by the next

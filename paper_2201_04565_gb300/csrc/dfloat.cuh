@@ -374,8 +374,8 @@ __device__ __forceinline__ bool ff_gt_un(ff a, ff b)
 // (relative error below 2^-22.9), the residual rho = 1 - r^2 y0^2, and one
 // double-float Newton step, r0 / r = r0 y0 (1 + rho / 2), whose neglected
 // term 3/8 rho^2 would reach 2^-45.2 and is kept as a factor 1 + 3/4 rho on rho
-// (in eight springs' sum the force's error falls from 1.9e-14 to 7e-15 k r0, root
-// mean square). With y0^2 = q + qe exactly (TwoProd),
+// (in the sum of eight springs the error of all g falls from 2.8e-14 to 1.2e-14 k r0,
+// root mean square). With y0^2 = q + qe exactly (TwoProd),
 // rho is three fused multiply-adds: 1 - r2.hi q is formed exactly before
 // its one rounding (r2.hi q lies within about 2^-21.9 of 1), then the terms
 // r2.hi qe and r2.lo q of order 2^-24 follow (r2.lo qe, below 2^-47, is

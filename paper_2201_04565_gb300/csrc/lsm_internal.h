@@ -69,23 +69,35 @@ inline double max_critical_length(const std::vector<SpringType> &types)
 
 // The DF force split (tile_body.cuh): forces are held as a multiple of a unit u
 // plus a remainder below u / 2, so that the multiples of a particle's forces
-// (`terms` at most) add without rounding while each is at most 2^24 u / terms. u is
-// the power of two that takes 1.5 times the largest tensile force of any type
-// (k (rc - r0), or 1/32 of k r0) into that range; a spring with |k (1 - r0/r)| up to
-// cmax stays in it (0 if no such limit exists: an unbreakable type).
+// (`terms` at most) add without rounding while each is at most 2^24 u / terms.
+// The remainders are floats, so a force is exact to some 2^-24 u: u is the smaller
+// of two powers of two,
+//   - the one that takes 1.5 times the largest tensile force of any type
+//     (k (rc - r0), or 1/32 of k r0) into that range, and
+//   - 2^-21.5 (3D: 2^-22) of the least k r0 of any type. At this line the sum of
+//     eight springs (18) is off by 2.2e-14 (3.1e-14) k r0, root mean square, against 2.8e-14
+//     (3.7e-14) of a plain double-float sum without the second-order term of 1 - r0/r,
+//     and by half of that from 1 - r0/r alone. Without the line the forces
+//     of a soft phase lose a factor of its contrast: 3e-12 k r0 at 1,000, single
+//     precision at 1e6.
+// A spring with |k (1 - r0/r)| up to cmax stays in the exact range (0 if no such
+// limit exists: an unbreakable type); one above it is summed with error terms, with
+// no loss.
 struct DfSplit {
     double unit = 0x1p-21, cmax = 0.0;
 };
 inline DfSplit df_split(const std::vector<SpringType> &types, int terms)
 {
-    double f = 0.0, rc = 1.0;
+    double f = 0.0, rc = 1.0, soft = INFINITY;
     for (const SpringType &t : types) {
         const double r = std::sqrt(t.rc2);
         rc = std::fmax(rc, r);
         f = std::fmax(f, t.k * std::fmax(std::isfinite(r) ? r - t.r0 : 0.0, 0.03125 * t.r0));
+        if (t.k > 0.0) soft = std::fmin(soft, t.k * t.r0);
     }
     DfSplit s;
     s.unit = std::exp2(std::ceil(std::log2(f > 0.0 ? 1.5 * f * terms : 1.0)) - 24.0);
+    if (std::isfinite(soft)) s.unit = std::fmin(s.unit, std::exp2(std::floor(std::log2(soft) - (terms > 8 ? 22.0 : 21.5))));
     s.cmax = std::isfinite(rc) ? s.unit * 0x1p24 / terms / rc : 0.0;
     return s;
 }
