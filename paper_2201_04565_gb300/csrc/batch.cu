@@ -651,7 +651,7 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     b.fix_S = std::min(61 - (int)std::ceil(std::log2(extent)), 47 - (int)std::ceil(std::log2(b.a * std::sqrt(2.0))));
     b.fix_S = std::min(b.fix_S, 47 - (int)std::floor(std::log2(max_critical_length(h0.types))));
     b.a_fix = std::llround(std::ldexp(b.a, b.fix_S));
-    b.df = df_split(h0.types, 8);
+    b.df = df_split(h0.types, 4, 4);
     for (int q = 0; q < 2; q++) {
         BT_TRY(balloc(&b.X[q], 2 * NP));
         BT_TRY(balloc(&b.VH[q], 2 * NP));

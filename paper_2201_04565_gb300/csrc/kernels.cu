@@ -608,7 +608,7 @@ static cudaError_t upload_tile(Ctx &c)
     c.fix_S = std::min(c.fix_S, 47 - (int)std::floor(std::log2(max_critical_length(h.types))));
     c.a_fix = std::llround(std::ldexp(h.a, c.fix_S));
     c.h_fix = std::llround(std::ldexp(hrow, c.fix_S));
-    c.df = df_split(h.types, 8);
+    c.df = c.tri ? df_split(h.types, 2, 4) : df_split(h.types, 4, 4);
     std::vector<int64_t> sbase(np, 0);
     for (int64_t s = h.m - 1; s >= 0; s--) sbase[c.tgidx[h.si[s]]] = s;
     std::vector<TypeDF> tdf(h.types.size());

@@ -68,37 +68,82 @@ inline double max_critical_length(const std::vector<SpringType> &types)
 }
 
 // The DF force split (tile_body.cuh): forces are held as a multiple of a unit u
-// plus a remainder below u / 2, so that the multiples of a particle's forces
-// (`terms` at most) add without rounding while each is at most 2^24 u / terms.
+// plus a remainder below u / 2, so that the multiples of a particle's forces add
+// without rounding while those forces sum to 2^24 u at most.
 // The remainders are floats, so a force is exact to some 2^-24 u: u is the smaller
 // of two powers of two,
-//   - the one that takes 1.5 times the largest tensile force of any type
-//     (k (rc - r0), or 1/32 of k r0) into that range, and
+//   - the one that takes 1.5 times the largest tensile forces (k (rc - r0), or 1/32
+//     of k r0) of all springs of a particle into that range, and
 //   - 2^-21.5 (3D: 2^-22) of the least k r0 of any type. At this line the sum of
 //     eight springs (18) is off by 2.2e-14 (3.1e-14) k r0, root mean square, against 2.8e-14
 //     (3.7e-14) of a plain double-float sum without the second-order term of 1 - r0/r,
 //     and by half of that from 1 - r0/r alone. Without the line the forces
 //     of a soft phase lose a factor of its contrast: 3e-12 k r0 at 1,000, single
 //     precision at 1e6.
-// A spring with |k (1 - r0/r)| up to cmax stays in the exact range (0 if no such
-// limit exists: an unbreakable type); one above it is summed with error terms, with
-// no loss.
+// Intact springs with |k (1 - r0/r)| up to cmax (df_cmax) stay in the exact range;
+// a particle with one above it is summed with error terms, with no loss.
 struct DfSplit {
     double unit = 0x1p-21, cmax = 0.0;
 };
-inline DfSplit df_split(const std::vector<SpringType> &types, int terms)
+
+// The longest sum of the forces on one particle, n0 of its springs of shell 0 and n1
+// of shell 1, by the types that touch its phase (types: [phase][phase][shell]).
+template <typename FORCE>
+double df_longest(const std::vector<SpringType> &types, int n0, int n1, FORCE force)
 {
-    double f = 0.0, rc = 1.0, soft = INFINITY;
-    for (const SpringType &t : types) {
-        const double r = std::sqrt(t.rc2);
-        rc = std::fmax(rc, r);
-        f = std::fmax(f, t.k * std::fmax(std::isfinite(r) ? r - t.r0 : 0.0, 0.03125 * t.r0));
-        if (t.k > 0.0) soft = std::fmin(soft, t.k * t.r0);
+    const size_t np = (size_t)std::lround(std::sqrt(0.5 * (double)types.size()));
+    double most = 0.0;
+    for (size_t p = 0; p < np; p++) {
+        double f[2] = {0.0, 0.0};
+        for (size_t q = 0; q < np; q++)
+            for (int s = 0; s < 2; s++)
+                f[s] = std::fmax(f[s], std::fmax(force(types[(p * np + q) * 2 + s]), force(types[(q * np + p) * 2 + s])));
+        most = std::fmax(most, n0 * f[0] + n1 * f[1]);
     }
+    return most;
+}
+
+// The largest c for which intact springs with |k (1 - r0/r)| <= c sum to less than
+// `range`. Compressed (r < r0) such a spring's force is at most c r0; stretched
+// r <= r0 k / (k - c) and r <= rc, so it is at most the smaller of
+// c r0 k / (k - c) and k (rc - r0). (rc alone as the bound on r takes a soft type's
+// long rc for the stiff one's force: with critical strains of 0.05 and 0.3 the
+// stiff phase would leave the range at a strain of 0.035.)
+inline double df_cmax(const std::vector<SpringType> &types, int n0, int n1, double range)
+{
+    auto longest = [&](double c) {
+        return df_longest(types, n0, n1, [c](const SpringType &t) {
+            if (!(t.k > 0.0)) return 0.0;
+            const double pull = t.k * std::fmax(std::sqrt(t.rc2) - t.r0, 0.0);
+            const double grow = c < t.k ? c * t.r0 * (t.k / (t.k - c)) : INFINITY;
+            return std::fmax(c * t.r0, std::fmin(pull, grow));
+        });
+    };
+    double lo = 0.0, hi = INFINITY;
+    for (const SpringType &t : types)
+        if (t.k > 0.0) hi = std::fmin(hi, range / t.r0);  // one spring's force already
+    if (!std::isfinite(hi)) return 0.0;                   // no force at all
+    for (int i = 0; i < 50; i++) {
+        const double c = 0.5 * (lo + hi);
+        (longest(c) < range ? lo : hi) = c;
+    }
+    return lo;
+}
+
+// n0, n1: springs of a particle in the types' shells 0 and 1.
+inline DfSplit df_split(const std::vector<SpringType> &types, int n0, int n1)
+{
+    const double f = df_longest(types, n0, n1, [](const SpringType &t) {
+        const double r = std::sqrt(t.rc2);
+        return t.k * std::fmax(std::isfinite(r) ? r - t.r0 : 0.0, 0.03125 * t.r0);
+    });
+    double soft = INFINITY;
+    for (const SpringType &t : types)
+        if (t.k > 0.0) soft = std::fmin(soft, t.k * t.r0);
     DfSplit s;
-    s.unit = std::exp2(std::ceil(std::log2(f > 0.0 ? 1.5 * f * terms : 1.0)) - 24.0);
-    if (std::isfinite(soft)) s.unit = std::fmin(s.unit, std::exp2(std::floor(std::log2(soft) - (terms > 8 ? 22.0 : 21.5))));
-    s.cmax = std::isfinite(rc) ? s.unit * 0x1p24 / terms / rc : 0.0;
+    s.unit = std::exp2(std::ceil(std::log2(f > 0.0 ? 1.5 * f : 1.0)) - 24.0);
+    if (std::isfinite(soft)) s.unit = std::fmin(s.unit, std::exp2(std::floor(std::log2(soft) - (n0 + n1 > 8 ? 22.0 : 21.5))));
+    s.cmax = df_cmax(types, n0, n1, s.unit * (0x1p24 - 0x1p14));  // less what rounding adds
     return s;
 }
 

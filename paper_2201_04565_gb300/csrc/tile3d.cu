@@ -648,7 +648,7 @@ cudaError_t tile3_upload(Ctx &c)
     c.fix_S = std::min(c.fix_S, 47 - (int)std::ceil(std::log2(h.a * std::sqrt(2.0))));
     c.fix_S = std::min(c.fix_S, 47 - (int)std::floor(std::log2(max_critical_length(h.types))));
     c.a_fix = std::llround(std::ldexp(h.a, c.fix_S));
-    c.df = df_split(h.types, 18);
+    c.df = df_split(h.types, 6, 12);
     const double aa = std::ldexp((double)c.a_fix, -c.fix_S);
     std::vector<TypeDF> tdf(h.types.size());
     for (size_t q = 0; q < h.types.size(); q++) {

@@ -117,7 +117,7 @@ struct TileArgs {
     double hrow;               // triangular packing: row height
     float p24, p0;             // 2^(24-S), 2^-S
     unsigned df_bias;          // DF: f2d_force_scaled bias for forces held in units of p24
-    float df_M, df_cmax;       // DF: the force split's 1.5 2^23 u (in those units), and the c it is exact for
+    float df_M, df_cmax;       // DF: the force split's 1.5 2^23 u (in those units), and the range of its plain sums
     double dt, hdt, gamma, a;
     int grip_mode;
     int rate_on;               // constant strain rate: grips at rate_eps0 + (s - rate_step0) rate_dt
@@ -149,10 +149,10 @@ __host__ __device__ constexpr int tile_min_ctas()
 
 // Sum of a particle's DF spring forces in the canonical order. A force is held
 // split (ff_mul_split): f = lo - hi, hi a multiple of the context's unit u. While
-// every |hi| is within the split's range (df_split), the sums of all of them are
-// exact in float, and the low parts, below u, are summed in float beside them: two
-// additions per term (DfSum). A spring compressed beyond that (the springs'
-// "big" flag) takes the cascaded sum (Ogita, Rump and Oishi, 2005) of the same
+// the springs' factors are within the split's range (df_split), the sums of the high
+// parts are exact in float, and the low parts, below u, are summed in float beside
+// them: two additions per term (DfSum). A spring with a factor beyond it ("big")
+// takes the cascaded sum (Ogita, Rump and Oishi, 2005) of the same
 // terms, a TwoSum chain over the high parts (DfSumCareful): where no high sum
 // rounds, its errors are 0 and both give the same bits, so kernels may decide
 // it per warp, per block or always. value(): the sum as a double (exact
