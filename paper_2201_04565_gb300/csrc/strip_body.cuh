@@ -440,7 +440,7 @@ __device__ __forceinline__ void strip_run(const TileArgs &A, int R, int sx, int 
         const bool sum_springs = SAMPLE && own && owner;
         FT f0x, f0y, f1x, f1y, f2x, f2y, f3x{}, f3y{};
         int s0, s1, s2, s3 = S_NONE;
-        bool big = false;  // DF: a force beyond the split's exact range
+        bool big = !TEST;  // DF: a force beyond the split's exact range (tile_body.cuh)
         if constexpr (PREC == LSM_PREC_DF && !SAMPLE && TEST) {
             // two springs at a time on packed instructions (the same bits)
             if constexpr (LAT == 0) {

@@ -218,7 +218,9 @@ __device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, 
                                             int ep, int pp, uint16_t mk, const long long (&xp)[3], DfSumCareful (&F)[3],
                                             uint16_t &newb)
 {
-    bool big = PREC != LSM_PREC_DF;  // F32's forces are plain floats: always with error terms
+    // F32's forces are plain floats, and without a break test springs longer than the
+    // range allows for may be there: always with error terms
+    bool big = PREC != LSM_PREC_DF || !TEST;
 #pragma unroll 1
     for (int s = 0; s < 9; s++) {
         const int o = soff[s], ei = ep - o, eo = ep + o, sh = A.ssh[s] - 1;

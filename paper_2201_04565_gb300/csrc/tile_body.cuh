@@ -543,7 +543,9 @@ __device__ __forceinline__ void tile_body(const TileArgs &A, int bx, int by, int
     // 2a. forward springs of the owned particles
     using AT = typename std::conditional<FIX, ff, double>::type;  // per-thread sample sums
     AT w_acc{}, u_acc{};
-    bool big = false;  // DF: a force beyond the split's exact range
+    // DF: a force beyond the split's exact range; without a break test springs longer
+    // than the range allows for may be there
+    bool big = MODE != T_STEP;
     constexpr int dq[4] = {1, RX - 1, RX, RX + 1};
 #pragma unroll
     for (int k = 0; k < TY / NW; k++) {

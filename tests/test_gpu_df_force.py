@@ -107,3 +107,36 @@ def test_soft_phase_of_a_batch(L, sched, steps):
         rms, most = _error(topo[q], xs[q], b.state(q)[1], steps, k[1, 1], xs[q].shape[1])
         assert rms <= RMS and most <= MAX
     b.close()
+
+
+@pytest.mark.parametrize("kw,stretch", [(dict(path=0), 2.03), (dict(path=3), 2.03), (dict(lattice=1), 3.5), ("batch", 2.03)])
+def test_forces_of_springs_beyond_their_critical_length(L, kw, stretch):
+    """A soft sheet folded over and stretched beyond its critical strain by set_state:
+    the springs hold until the next step tests them, so the initial acceleration has
+    six springs of a particle on the fold pulling one way, more together than any
+    intact ones. All break in the step: v is dt / 2 times the force before it."""
+    k, e = _tables(10.0, 0.3)
+    img = np.full((30, 41), 2, np.uint8)
+    img[0, 0] = 1
+    g = L.Specimen.from_image(img, k, e, precision="exact64", **({} if kw == "batch" else dict(lattice=kw.get("lattice", 0))))
+    topo, X = g.topology(), g.state()[0]
+    g.close()
+    fold = 20.25 if "lattice" in kw else 20.0  # no two sites of a row onto one point
+    x = stretch * np.stack([np.abs(X[0] - fold), X[1]])
+    x += np.random.default_rng(3).uniform(-5e-3, 5e-3, x.shape)
+    x = np.round((x + 8.0) * 2.0 ** 34) / 2.0 ** 34
+    if kw == "batch":
+        from paper_2201_04565_gb300 import batch as B
+        s = B.Batch([img], k, e, precision="df64", dt=DT, damping=0.0)
+        s.set_state(0, x, np.zeros_like(x))
+        s.step(1)
+        v, broken = s.state(0)[1], s.broken(0)[0]
+    else:
+        s = L.Specimen.from_image(img, k, e, precision="df64", dt=DT, damping=0.0, **kw)
+        s.set_state(x, np.zeros_like(x))
+        s.step(1)
+        v, broken = s.state()[1], s.broken()[0]
+    s.close()
+    assert broken.all()
+    rms, most = _error(topo, x, 2.0 * v, 1, k[1, 1], x.shape[1])
+    assert rms <= 10 * RMS and most <= 10 * MAX  # the forces are ten times those of small strains
