@@ -8,16 +8,17 @@
 //      writes the block's own drifted positions, x(t+dt);
 //   2. compacts the block's particles into a list in raster order (porous
 //      volumes leave most voxels void; the list keeps every warp busy);
-//   3. for each listed particle evaluates all 18 of its springs, incoming springs by
-//      ascending source, then outgoing springs by ascending target (the
-//      canonical order of the sequential sum), accumulating the force in
-//      registers. Every spring is evaluated by both endpoints from the same
-//      data (d = x_upper - x_lower, the upper endpoint negates the force), so
-//      both see the same break decision and equal and opposite forces; the
-//      lower endpoint records breaks. No shared-memory force exchange and one
-//      barrier per step: in 3D that exchange (9 slots x 3 components per
-//      source voxel) would cost more shared memory than the recomputation
-//      costs arithmetic in these modes;
+//   3. for each listed particle evaluates all 18 of its springs slot by slot
+//      (forward offsets by ascending target), the incoming spring then the
+//      outgoing one, accumulating the force in registers: not the canonical
+//      order of the sequential sum, but the same in every step, so that the
+//      states do not depend on how the steps are grouped into calls. Every
+//      spring is evaluated by both endpoints from the same data (d = x_upper
+//      - x_lower, the upper endpoint negates the force), so both see the same
+//      break decision and equal and opposite forces; the lower endpoint
+//      records breaks. No shared-memory force exchange: in 3D that (9 slots x
+//      3 components per source voxel) would cost more shared memory than the
+//      recomputation costs arithmetic in these modes;
 //      and integrates (Eqs. 4-5) in FP64, writing vh(t+3dt/2).
 // The FP64 modes keep the spring-list kernels for 3D: recomputing every
 // spring twice would double their FP64-pipe work.
@@ -181,23 +182,23 @@ __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl,
             u = ff_add_sloppy(u, ff_mul(ff_mul_f(t.k, 0.5f), ff_sqr(st)));
             w = ff_add_sloppy(w, ff_mul(d[0], df_pair(f[0])));
         }
-    } else {  // F32: e = d - o exact, (2 o + e).e carries no cancellation
+    } else {  // F32: e = d - o exact, (2 o + e).e carries no cancellation; the operations of spring_f32_pair
         float e[3], dd[3], num = t.cor.hi;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             const long long ef = du[c] - dl[c] - (long long)A.sd[s][c] * A.a_fix;
             e[c] = fix_to_float_i2f(ef, A.p24, A.p0);
             const float o = A.sd[s][c] == 0 ? 0.0f : (A.sd[s][c] > 0 ? A.fa : -A.fa);
-            dd[c] = o + e[c];
-            num = fmaf(2.0f * o + e[c], e[c], num);
+            dd[c] = __fadd_rn(o, e[c]);
+            num = __fmaf_rn(__fmaf_rn(o, 2.0f, e[c]), e[c], num);
         }
-        const float r2f = A.oo2[A.ssh[s] - 1] + num;
+        const float r2f = __fadd_rn(A.oo2[A.ssh[s] - 1], num);
         if (TEST && r2f > t.rc2.hi) return false;
-        const float ir = rsqrtf(r2f);
-        const float st = __fdividef(num, fmaf(r2f, ir, t.r0.hi));  // r - r0
-        const float cc = t.k.hi * st * ir;
+        const float ir = rsqrt_approx(r2f);
+        const float st = __fdividef(num, __fmaf_rn(r2f, ir, t.r0.hi));  // r - r0
+        const float cc = __fmul_rn(__fmul_rn(t.k.hi, st), ir);
 #pragma unroll
-        for (int c = 0; c < 3; c++) f[c] = ff{-(cc * dd[c]), 0.0f};  // in the form of a split force
+        for (int c = 0; c < 3; c++) f[c] = ff{-__fmul_rn(cc, dd[c]), 0.0f};  // in the form of a split force
         if (sample) {
             u = ff_add_f(u, 0.5f * t.k.hi * st * st);
             w = ff_add_f(w, dd[0] * -f[0].hi);
@@ -208,7 +209,10 @@ __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl,
 
 // The 18 springs of a particle: forces into F (split sums), new breaks of its
 // forward springs into newb; slot s's incoming spring is broken by its source's
-// flags or its own break test, which the source's thread records. In DF the sums
+// flags or its own break test, which the source's thread records. Slot by slot, the
+// incoming spring then the outgoing one: they share offset, shell and lattice vector.
+// (Pairs in the canonical order, all incoming springs first, took the 256^3 foam
+// from 755 to 781 us a step, in F32 from 697 to 770.) In DF the sums
 // go without error terms until a factor above cmax turns up (up to then every
 // partial sum is exact, see DfSum), and with them from there on. (Running all 18
 // springs again with error terms instead took the 256^3 foam from 754 to 970 us
@@ -391,33 +395,31 @@ k_tile3d(Tile3Args A)
             // springs side by side on packed instructions
             tile3_pairs<PREC, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb);
         } else {
-            // incoming by ascending source (descending slot), then outgoing
-#pragma unroll 1
-            for (int s = 8; s >= 0; s--) {
-                const int eq = ep - soff[s];
-                const int pq = S.ph[eq];
-                if (!pq || ((S.mk[eq] >> s) & 1)) continue;
-                const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
-                const TypeDF t = sdf[(((pq - 1) * A.nphase) + (pp - 1)) * 2 + (A.ssh[s] - 1)];
-                ff f[3], wd{0.0f, 0.0f}, ud{0.0f, 0.0f};
-                if (!spring3<PREC, MODE == T_STEP>(A, xq, xp, s, t, f, wd, ud, false)) continue;
-#pragma unroll
-                for (int c = 0; c < 3; c++) F3[c].sub(f[c]);
-            }
+            // the same springs in the same order, one at a time
 #pragma unroll 1
             for (int s = 0; s < 9; s++) {
-                const int eq = ep + soff[s];
-                const int pq = S.ph[eq];
-                if (!pq || ((mk >> s) & 1)) continue;
-                const long long xq[3] = {S.xf[0][eq], S.xf[1][eq], S.xf[2][eq]};
-                const TypeDF t = sdf[(((pp - 1) * A.nphase) + (pq - 1)) * 2 + (A.ssh[s] - 1)];
-                ff f[3];
-                if (!spring3<PREC, MODE == T_STEP>(A, xp, xq, s, t, f, w_acc, u_acc, SAMPLE)) {
-                    newb |= (uint16_t)(1u << s);
-                    continue;
-                }
+                const int sh = A.ssh[s] - 1, ei = ep - soff[s], eo = ep + soff[s];
+                const int pi = S.ph[ei], po = S.ph[eo];
+                if (pi && !((S.mk[ei] >> s) & 1)) {
+                    const long long xq[3] = {S.xf[0][ei], S.xf[1][ei], S.xf[2][ei]};
+                    const TypeDF t = sdf[(((pi - 1) * A.nphase) + (pp - 1)) * 2 + sh];
+                    ff f[3], wd{0.0f, 0.0f}, ud{0.0f, 0.0f};
+                    if (spring3<PREC, MODE == T_STEP>(A, xq, xp, s, t, f, wd, ud, false)) {
 #pragma unroll
-                for (int c = 0; c < 3; c++) F3[c].add(f[c]);
+                        for (int c = 0; c < 3; c++) F3[c].sub(f[c]);
+                    }
+                }
+                if (po && !((mk >> s) & 1)) {
+                    const long long xq[3] = {S.xf[0][eo], S.xf[1][eo], S.xf[2][eo]};
+                    const TypeDF t = sdf[(((pp - 1) * A.nphase) + (po - 1)) * 2 + sh];
+                    ff f[3];
+                    if (spring3<PREC, MODE == T_STEP>(A, xp, xq, s, t, f, w_acc, u_acc, SAMPLE)) {
+#pragma unroll
+                        for (int c = 0; c < 3; c++) F3[c].add(f[c]);
+                    } else {
+                        newb |= (uint16_t)(1u << s);
+                    }
+                }
             }
         }
         if (MODE == T_STEP && newb) {
