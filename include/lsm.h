@@ -76,9 +76,9 @@ typedef enum {
  *      step's range check as LSM_ENONFINITE. For image builds DF and F32 run on the 2D strip or
  *      tile kernels (square lattice), the strip kernel (triangular
  *      packing), the 3D voxel tile kernel, or (path 1) the spring-list
- *      kernels with the same fixed-point spring vectors. Their sums go in
- *      canonical spring order in 2D, slot by slot on the voxel kernel; the
- *      states do not depend on how the steps are grouped into calls.
+ *      kernels with the same fixed-point spring vectors. The voxel kernel
+ *      sums a particle's springs offset by offset, the incoming one then the
+ *      outgoing one, in every step.
  *      Network builds have no lattice vectors:
  *      there F32 forms the spring vector in double and DF runs as
  *      LSM_PREC_FAST64. */

@@ -636,7 +636,7 @@ static cudaError_t upload_tile(Ctx &c)
     }
     LSM_TRY(dalloc(&c.tvobs, 2 * np));
     LSM_TRY(dalloc(&c.tph, np));
-    LSM_TRY(dalloc(&c.tmask, np));
+    LSM_TRY(dalloc(&c.tmask, tile_mask_bytes(np)));
     LSM_TRY(dalloc(&c.tbrk, 4 * np));
     LSM_TRY(dalloc(&c.tmass, h.nphase));
     LSM_TRY(dalloc(&c.tinvm, 4 * h.nphase));
@@ -655,7 +655,7 @@ static cudaError_t upload_tile(Ctx &c)
     }
     LSM_TRY(cudaMemsetAsync(c.tvobs, 0, 2 * np * sizeof(double), st));
     LSM_TRY(cudaMemcpyAsync(c.tph, gph, np, cudaMemcpyHostToDevice, st));
-    LSM_TRY(cudaMemsetAsync(c.tmask, 0, np, st));
+    LSM_TRY(cudaMemsetAsync(c.tmask, 0, tile_mask_bytes(np), st));
     LSM_TRY(cudaMemsetAsync(c.tbrk, 0xff, 4 * np * sizeof(long long), st));
     LSM_TRY(cudaMemcpyAsync(c.tmass, mtab.data(), h.nphase * sizeof(double), cudaMemcpyHostToDevice, st));
     LSM_TRY(cudaMemcpyAsync(c.tinvm, itab.data(), 4 * h.nphase * sizeof(double), cudaMemcpyHostToDevice, st));

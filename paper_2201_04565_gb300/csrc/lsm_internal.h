@@ -216,6 +216,11 @@ struct MultiPlan {
 };
 MultiPlan multi_shape(int prec, int nx, int ny);
 
+// Bytes of the 2D grid's broken flags, one per cell: whole 32-bit words, because the
+// multi-step kernel sets a cell's flags by an atomic on the aligned word that holds
+// them.
+inline size_t tile_mask_bytes(int64_t np) { return ((size_t)np + 3) & ~(size_t)3; }
+
 
 struct Ctx {
     HostNet h;  // host copy of topology (kept for queries and rebuilds)

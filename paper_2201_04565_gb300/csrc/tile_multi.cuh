@@ -263,7 +263,7 @@ __device__ __forceinline__ void tile_multi_body(const TileArgs &A, int bx, int b
             nb <<= grp * NS;
             mk |= nb;
             if (own) {
-                // the groups of a cell share its flag byte
+                // the groups of a cell share its flag byte (tile_mask_bytes: whole words)
                 const uintptr_t a = (uintptr_t)(A.mask + g);
                 atomicOr((unsigned *)(a & ~(uintptr_t)3), nb << (8 * (a & 3)));
 #pragma unroll
