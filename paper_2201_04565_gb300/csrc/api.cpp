@@ -550,6 +550,23 @@ lsm_status lsm_get_state(lsm_ctx *c, double *x, double *v)
     lsm_status st = device_status(c);
     if (st != LSM_OK) return st;
     cudaError_t e = cudaSuccess;
+    if (c->tile && c->n != c->tnp && c->tnp <= lsm::STATE_HOST_CELLS) {  // whole grids, picked here
+        const size_t dg = (size_t)c->dim * c->tnp;
+        std::vector<double> g((x ? dg : 0) + (v ? dg : 0));
+        double *gx = g.data(), *gv = gx + (x ? dg : 0);
+        if (x) e = cudaMemcpyAsync(gx, c->tx[c->tcur], dg * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess && v)
+            e = cudaMemcpyAsync(gv, c->tvobs, dg * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess) return cuda_fail(c, e, "get_state");
+        for (int cc = 0; cc < c->dim; cc++)
+            for (int64_t p = 0; p < c->n; p++) {
+                const int64_t q = cc * c->tnp + c->tgidx[p];
+                if (x) x[cc * c->n + p] = gx[q];
+                if (v) v[cc * c->n + p] = gv[q];
+            }
+        return LSM_OK;
+    }
     if (c->tile) {
         if (x) e = lsm::tile_state(*c, c->tx[c->tcur], x);
         if (e == cudaSuccess && v) e = lsm::tile_state(*c, c->tvobs, v);

@@ -377,6 +377,11 @@ void prefault(void *p, size_t bytes) noexcept;
 // Tile paths: a grid array [dim][tnp] to host memory [dim][n], the particles
 // in canonical order (the copies are enqueued on the context's stream).
 cudaError_t tile_state(Ctx &c, const double *grid, double *host);
+// Grids with empty cells of up to this many go to the host whole and are picked
+// there: the packing's launch and copy for each component cost more than the cells
+// (x and v, whole and packed: 64 x 64 cells 42 and 78 us, 160 x 128 80 and 77, 200 x 150
+// 104 and 78; 24^3 84 and 105, 30^3 124 and 105).
+constexpr int64_t STATE_HOST_CELLS = 20480;
 cudaError_t launch_steps(Ctx &c, int64_t nsteps, bool record);
 cudaError_t launch_apply_strain(Ctx &c, double eps_old, double eps_new);
 cudaError_t launch_observe(Ctx &c, DeviceSample *dst);
