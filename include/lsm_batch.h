@@ -61,8 +61,9 @@ lsm_status lsm_batch_autotune(lsm_batch *b, int32_t steps_per_trial, int32_t *ti
  * increments keep 16-row tiles; the states are the same bits either way.
  * grid >= 0 (tiles only); order 0 or 1. LSM_EINVAL otherwise. A new batch
  * starts with strips (-16 where those outnumber the warps the device holds
- * at once, in DF mode; in F32 mode -8 from two thirds of these warps on, -16
- * above them) or 8-row tiles, largest specimens first, grid 0. */
+ * at once; in F32 mode also -8 from two thirds of these warps on, where the
+ * specimens' widths suit strips) or 8-row tiles (F32: 16 rows from three per
+ * SM on), largest specimens first, grid 0. */
 lsm_status lsm_batch_set_schedule(lsm_batch *b, int32_t tile_y, int32_t grid, int32_t order);
 
 /* Load increment of every specimen to the absolute strains eps[0..count-1]

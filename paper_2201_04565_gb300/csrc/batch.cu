@@ -391,6 +391,13 @@ static int64_t batch_strips(const BatchCtx &b, int R)
     return n;
 }
 
+static int64_t batch_tiles(const BatchCtx &b, int rows)
+{
+    int64_t n = 0;
+    for (int s = 0; s < b.S; s++) n += (int64_t)((b.nx[s] + 31) / 32) * ((b.ny[s] + rows - 1) / rows);
+    return n;
+}
+
 // Rows per strip of the 16-row schedule: 16, or, where strips of 16 rows take
 // more than one wave of the resident warps and strips of up to 64 rows only
 // one, the least rows for one wave: a second wave that is partly empty costs
@@ -748,16 +755,20 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     // autotuner picks on the benchmark's batches; a warp sweeping a strip is
     // latency-bound when few run), 8-row tiles otherwise (12 specimens of
     // 128^2, a step: exact 37.4 -> 35.4 us against 16 rows, df64 11.3 -> 10.7,
-    // f32 12.3 -> 10.1). F32 sweeps pay from two thirds of the warps on, as
-    // in the single-specimen kernel, then on 8-row strips (12 specimens of
-    // sides 32 to 512: 38.2 us on tiles, 29.7 on strips).
+    // f32 12.3 -> 10.1). F32: 16-row tiles where they are three per SM, as in the
+    // single-specimen kernel (6 of 200^2, 546 tiles: 14.0 us with 8 rows, 12.0 with
+    // 16; 5 of 200^2, 455: 10.3 and 10.8); sweeps pay from two thirds of the warps
+    // on, where strips of 8 rows are fewer than 2.4 per 16-row tile, then on 8-row
+    // strips (12 specimens of sides 32 to 512: 35.0 us on tiles, 29.7 on strips; a
+    // specimen of 64 columns takes three strips for two tiles: 200 of 64^2 29.3 us on
+    // strips, 25.0 on tiles).
     const int64_t slots = batch_strips_ok(b) ? batch_strip_slots() : 0;
-    int ty = 8;
-    if (slots > 0 && b.prec == LSM_PREC_F32) {
-        const int64_t n8 = batch_strips(b, 8);
-        if (3 * n8 >= 2 * slots) ty = n8 <= slots ? -8 : -16;
-    } else if (slots > 0 && batch_strips(b, 16) >= slots) {
-        ty = -16;
+    const bool fill = slots > 0 && batch_strips(b, 16) >= slots;
+    int ty = fill ? -16 : 8;
+    if (b.prec == LSM_PREC_F32 && !fill) {
+        const int64_t n8 = batch_strips(b, 8), t16 = batch_tiles(b, 16);
+        if (t16 >= F32_TILES_16) ty = 16;
+        if (slots > 0 && 3 * n8 >= 2 * slots && 5 * n8 < 12 * t16) ty = n8 <= slots ? -8 : -16;
     }
     BT_TRY(build_tiles(b, ty, 1));
     // initial acceleration of every specimen (vh = v + dt/2 a(0))

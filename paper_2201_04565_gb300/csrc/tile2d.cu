@@ -128,9 +128,8 @@ constexpr int TILE_X = 32;
 // as 8-row tiles would need).
 // F32 steps take 8 rows where 16-row tiles are fewer than three per SM, and 16
 // where there are more (300^2 8.5 -> 6.5 us, 400^2 9.6 -> 7.9 us with 8 rows;
-// 500^2 10.8 us with 16 rows, 11.9 with 8).
+// 500^2 10.8 us with 16 rows, 11.9 with 8): F32_TILES_16 (tile_body.cuh).
 constexpr int TILE_Y_SAMPLE = 16;
-constexpr int64_t F32_TILES_16 = 3 * 152;
 template <int PREC, bool SAMPLE>
 constexpr int tile_y() { return (PREC == LSM_PREC_DF || PREC == LSM_PREC_EXACT64) && !SAMPLE ? 8 : TILE_Y_SAMPLE; }
 
