@@ -55,8 +55,9 @@ lsm_status lsm_batch_autotune(lsm_batch *b, int32_t steps_per_trial, int32_t *ti
 /* Set the schedule explicitly: tile_y 8, 16 or 32 (tiles of 32 columns and
  * that many rows, one CTA each), or -8, -16, -32 (F32 and DF modes, every
  * specimen below 2^29 pixels): the time steps run as one warp per strip of
- * 30 owned columns and 8, 16 or 32 rows (-16: up to 64 rows where that lets
- * the device hold all strips at once), the register-resident sweep of the
+ * 30 owned columns and 8, 16 or 32 rows (-16: up to 64 rows where the device
+ * then holds all strips at once and that is the faster by a measured rule on
+ * their number), the register-resident sweep of the
  * single-specimen strip kernel (sample sums per strip), while load
  * increments keep 16-row tiles; the states are the same bits either way.
  * grid >= 0 (tiles only); order 0 or 1. LSM_EINVAL otherwise. A new batch

@@ -400,17 +400,24 @@ static int64_t batch_tiles(const BatchCtx &b, int rows)
 
 // Rows per strip of the 16-row schedule: 16, or, where strips of 16 rows take
 // more than one wave of the resident warps and strips of up to 64 rows only
-// one, the least rows for one wave: a second wave that is partly empty costs
-// more than the longer sweeps (20 specimens of sides 32 to 512, 4,490 strips
-// of 16 rows for 3,040 warps: DF 77.5 us a step with
-// 16 rows, 71.4 in one wave; F32 57.6 and 50.7).
+// one, the least rows for one wave where that is the faster: a last wave that is
+// partly empty costs more than longer sweeps (20 specimens of sides 32 to 512, 4,490
+// strips of 16 rows for 3,040 warps: DF 77.5 us a step with 16 rows, 71.4 in one
+// wave; F32 57.6 and 50.7), but several waves run out of step and share the pipes
+// better (60 of 256^2, 2.84 waves: DF 131.9 us with 16 rows, 146.1 in one wave of
+// 52). Measured over 43 batches, in units of a row of a full wave (DF 2.73 us, F32
+// 1.87): one wave costs its rows and the two beside them, 0.16 less for each CTA of
+// the five that an SM does without; 16 rows cost 15.4 a wave and 4.8 (F32: 17.4
+// and 2.1).
 static int batch_strip_rows(const BatchCtx &b)
 {
-    const int64_t slots = batch_strip_slots();
-    if (slots == 0 || batch_strips(b, 16) <= slots || batch_strips(b, 64) > slots) return 16;
+    const int64_t slots = batch_strip_slots(), n16 = batch_strips(b, 16);
+    if (slots == 0 || n16 <= slots || batch_strips(b, 64) > slots) return 16;
     int R = 17;
     while (batch_strips(b, R) > slots) R++;
-    return R;
+    const int64_t ctas = (batch_strips(b, R) * STRIP_CTAS + slots - 1) / slots;  // per SM
+    const double one = (R + 2) * (1.0 - 0.16 * (double)(STRIP_CTAS - ctas)), waves = (double)n16 / (double)slots;
+    return one < (b.prec == LSM_PREC_F32 ? 17.4 * waves + 2.1 : 15.4 * waves + 4.8) ? R : 16;
 }
 
 // (Re)build the tile list for tile height ty and order (0 natural, 1 largest

@@ -24,9 +24,11 @@ def _per_step(b):
 
 
 # F32: on both sides of the tile height's line, many narrow specimens (three strips
-# for two tiles) and few wide ones; DF: more strips of 16 rows than twice the warps
-@pytest.mark.parametrize("precision,count,side", [("f32", 6, 200), ("f32", 5, 200), ("f32", 200, 64), ("f32", 24, 150)])
-def test_default_schedule_is_among_the_fastest(precision, count, side):
+# for two tiles) and few wide ones; strips of 16 rows for one to three times the warps
+@pytest.mark.parametrize("precision,count,side,bound", [("f32", 6, 200, 1.1), ("f32", 5, 200, 1.1), ("f32", 200, 64, 1.1),
+                                                        ("f32", 24, 150, 1.1), ("df64", 60, 256, 1.05),
+                                                        ("df64", 24, 256, 1.05), ("f32", 60, 256, 1.05)])
+def test_default_schedule_is_among_the_fastest(precision, count, side, bound):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -43,4 +45,4 @@ def test_default_schedule_is_among_the_fastest(precision, count, side):
         b.set_schedule(ty, 0, 1)
         others.append(_per_step(b))
     b.close()
-    assert default < 1.1 * min(others)
+    assert default < bound * min(others)
