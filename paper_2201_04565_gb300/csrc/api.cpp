@@ -39,8 +39,9 @@ static uintptr_t first_unmapped(uintptr_t lo, uintptr_t hi, uintptr_t page)
 
 void prefault(void *p, size_t bytes) noexcept
 {
-    // below malloc's mmap threshold a buffer comes from the heap and is mapped
-    if (!p || bytes < (128u << 10)) return;
+    // small buffers mostly come from the heap and are mapped: the look would cost more
+    // (2 to 3 us of a read of 25 to 45) than a fresh one's eight pages once
+    if (!p || bytes < (512u << 10)) return;
 #ifdef MADV_POPULATE_WRITE
     const long pg = sysconf(_SC_PAGESIZE);
     const uintptr_t page = pg > 0 ? (uintptr_t)pg : 4096, mask = ~(page - 1);

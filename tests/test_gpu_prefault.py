@@ -44,7 +44,7 @@ def test_mapped_buffer_costs_little(prefault, size, bound):
     assert (buf == 1).all()
 
 
-@pytest.mark.parametrize("size,touched", [(192 << 10, 0), (3 << 20, 0), (46 << 20, 9), (320 << 20, 4500)])
+@pytest.mark.parametrize("size,touched", [(576 << 10, 0), (3 << 20, 0), (46 << 20, 9), (320 << 20, 4500)])
 def test_fresh_buffer_is_mapped(prefault, size, touched):
     pages = size // mmap.PAGESIZE
     buf = mmap.mmap(-1, size, flags=mmap.MAP_PRIVATE | mmap.MAP_ANONYMOUS)
