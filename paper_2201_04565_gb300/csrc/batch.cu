@@ -774,7 +774,9 @@ static cudaError_t batch_upload(BatchCtx &b, const std::vector<HostNet> &nets, c
     int ty = fill ? -16 : 8;
     if (b.prec == LSM_PREC_F32 && !fill) {
         const int64_t n8 = batch_strips(b, 8), t16 = batch_tiles(b, 16);
-        if (t16 >= F32_TILES_16) ty = 16;
+        int sms = 0;
+        BT_TRY(device_sms(sms));
+        if (t16 >= F32_TILES_16 * sms) ty = 16;
         if (slots > 0 && 3 * n8 >= 2 * slots && 5 * n8 < 12 * t16) ty = n8 <= slots ? -8 : -16;
     }
     BT_TRY(build_tiles(b, ty, 1));

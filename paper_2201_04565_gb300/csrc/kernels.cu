@@ -571,6 +571,7 @@ static cudaError_t upload_tile(Ctx &c)
     c.tnp = np;
     c.tile_nphase = h.nphase;
     c.ntiles = c.tri ? 0 : tile_count(c);
+    LSM_TRY(device_sms(c.sms));
     if (c.strip) {
         bool fills = true;
         LSM_TRY(strip_geometry(c, &fills));
@@ -580,7 +581,7 @@ static cudaError_t upload_tile(Ctx &c)
         }
     }
     // path 2 keeps the one-step tile kernel
-    if (!c.strip && !c.tri && c.path_req != 2) c.multi = multi_shape(h.precision, h.nx, h.ny);
+    if (!c.strip && !c.tri && c.path_req != 2) c.multi = multi_shape(h.precision, h.nx, h.ny, c.sms);
     if (c.tri) c.ntiles = c.nstrips;  // the packing's samples all come from the strip kernel
     std::vector<double> X(2 * np);
     for (int64_t g = 0; g < np; g++) {

@@ -214,7 +214,16 @@ struct MultiPlan {
     int halo = 0;
     int64_t tiles = 0;
 };
-MultiPlan multi_shape(int prec, int nx, int ny);
+MultiPlan multi_shape(int prec, int nx, int ny, int sms);
+
+// SMs of the current device, for the rules that choose a kernel or a tile by how far
+// the tiles fill it.
+inline cudaError_t device_sms(int &sms)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e == cudaSuccess ? cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) : e;
+}
 
 // Bytes of the 2D grid's broken flags, one per cell: whole 32-bit words, because the
 // multi-step kernel sets a cell's flags by an atomic on the aligned word that holds
@@ -333,6 +342,7 @@ struct Ctx {
     std::map<int64_t, int64_t> graph_nodes;  // kernels per cached graph
     DfSplit df;                              // DF force split
     MultiPlan multi;                         // multi-step tile kernel (small 2D images)
+    int sms = 152;                           // SMs of the device (2D tile paths)
     std::map<int64_t, int> graph_buf;        // state buffer that a cached graph ends in
     std::map<int64_t, cudaGraphExec_t> graphs;
 };

@@ -213,7 +213,7 @@ static cudaError_t launch_tile_p(Ctx &c, TileArgs A)
     switch (c.h.precision) {
     case LSM_PREC_F32:
         if constexpr (MODE == T_STEP && !SAMPLE)
-            if (c.ntiles < F32_TILES_16) return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE, 8>(c, A);
+            if (c.ntiles < F32_TILES_16 * c.sms) return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE, 8>(c, A);
         return launch_tile<LSM_PREC_F32, MODE, SAMPLE, RATE>(c, A);
     case LSM_PREC_DF: return launch_tile<LSM_PREC_DF, MODE, SAMPLE, RATE>(c, A);
     default: return launch_tile<LSM_PREC_EXACT64, MODE, SAMPLE, RATE>(c, A);

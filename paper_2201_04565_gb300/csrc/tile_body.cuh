@@ -93,8 +93,8 @@ __device__ __forceinline__ double bmax_f(float v, double *sh)
 
 enum { T_STEP = 0, T_INIT = 1, T_OBSERVE = 2 };
 
-// 16-row tiles from which F32 steps take them, three per SM (tile2d.cu, batch.cu).
-constexpr int64_t F32_TILES_16 = 3 * 152;
+// 16-row tiles per SM from which F32 steps take them (tile2d.cu, batch.cu).
+constexpr int64_t F32_TILES_16 = 3;
 
 // Per-phase integration coefficients: vh' = c1 vh + c2 F is vh + dt (F - g vh)/m,
 // and c1h, c2h the same for a half step.

@@ -57,17 +57,16 @@ bool exact_mode(int prec) { return prec == LSM_PREC_EXACT64 || prec == LSM_PREC_
 //   four threads per cell, one spring each: 16 x 4 tiles up to one per two SMs
 //   (64^2: 11.3 -> 6.4 us; a halo of 2 with two threads per cell 6.7), then 32 x 4
 //   up to one per SM (100 x 90: 11.5 -> 8.6); 200 x 150 would lose (11.7, 16).
-MultiPlan multi_shape(int prec, int nx, int ny)
+MultiPlan multi_shape(int prec, int nx, int ny, int sms)
 {
-    constexpr int64_t SMS = 152;
     auto tiles = [&](int tx, int ty) { return (int64_t)((nx + tx - 1) / tx) * ((ny + ty - 1) / ty); };
     MultiPlan m;
     if (exact_mode(prec)) {
-        if (tiles(16, 4) <= SMS / 2) m = MultiPlan{MULTI_E16x4, 1, tiles(16, 4)};
-        else if (tiles(32, 4) <= SMS) m = MultiPlan{MULTI_E32x4, 1, tiles(32, 4)};
+        if (tiles(16, 4) <= sms / 2) m = MultiPlan{MULTI_E16x4, 1, tiles(16, 4)};
+        else if (tiles(32, 4) <= sms) m = MultiPlan{MULTI_E32x4, 1, tiles(32, 4)};
     } else {
-        if (tiles(16, 4) <= SMS + SMS / 16) m = MultiPlan{MULTI_16x4, 3, tiles(16, 4)};
-        else if (tiles(32, 8) <= 2 * SMS) m = MultiPlan{MULTI_32x8, 2, tiles(32, 8)};
+        if (tiles(16, 4) <= sms + sms / 16) m = MultiPlan{MULTI_16x4, 3, tiles(16, 4)};
+        else if (tiles(32, 8) <= 2 * sms) m = MultiPlan{MULTI_32x8, 2, tiles(32, 8)};
     }
     return m;
 }
