@@ -109,10 +109,10 @@ def algorithmic_bytes(n, m, dim):
 NCU_TRAFFIC = {
     # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum on three
     # time-step launches of each mode (the same 2048 x 2048 workload), mean
-    "df64": (238.5e6, "b85ff6edce8d"),
-    "f32": (238.4e6, "b85ff6edce8d"),
-    "fast64": (238.2e6, "b85ff6edce8d"),
-    "exact64": (238.0e6, "b85ff6edce8d"),
+    "df64": (238.4e6, "c79621137fb6"),
+    "f32": (238.3e6, "c79621137fb6"),
+    "fast64": (238.0e6, "c79621137fb6"),
+    "exact64": (238.1e6, "c79621137fb6"),
 }
 
 # Warp instructions executed by one time-step launch (ncu smsp__inst_executed.sum,
@@ -121,10 +121,10 @@ NCU_TRAFFIC = {
 # this gives the instruction-issue roofline, the one the fixed-point modes
 # are bound by.
 NCU_INSTRUCTIONS = {
-    "df64": (89419340, "b85ff6edce8d"),
-    "f32": (65048772, "b85ff6edce8d"),
-    "fast64": (314600626, "b85ff6edce8d"),
-    "exact64": (314600626, "b85ff6edce8d"),
+    "df64": (89419340, "c79621137fb6"),
+    "f32": (65048772, "c79621137fb6"),
+    "fast64": (314600626, "c79621137fb6"),
+    "exact64": (314600626, "c79621137fb6"),
 }
 
 # Binding unit of each mode's time-step kernel, from ncu on the same workload

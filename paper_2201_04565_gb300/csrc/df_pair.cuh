@@ -5,9 +5,10 @@
 // being FP32. sm_103a has add, mul and fma on pairs of floats (.f32x2): a packed
 // instruction takes the FMA pipe as long as its two scalar ones, but one issue
 // slot. spring_df_pair evaluates two springs side by side in the two halves;
-// every element goes through the operations of spring_df (tile_body.cuh; 3D: spring3,
-// tile3d.cu) in the same order with the same rounding, so both give the same bits. Differences
-// and negations are written as fma with -1, exact like the subtraction.
+// every element goes through the operations of spring_df (tile_body.cuh; 3D:
+// spring3, tile3d.cu) in the same order with the same rounding, so both give the
+// same bits. Differences and negations are written as fma with -1, exact like the
+// subtraction.
 // Together with the split force sums (DfSum) a 2048^2 step takes 89.1e6 warp
 // instructions instead of 108.8e6 and 112.1 us instead of 122.8, a 256^3 foam's
 // 830 us instead of 885 (775 on smaller blocks, tile3d.cu); what is left is

@@ -21,8 +21,9 @@
 // square root, so no tie arises). Products: the 106-bit integer product of
 // the significands, rounded with its round and sticky bits.
 //
-// Measured (EXACT64, one time step): 2048^2 composite on the tile kernel 1,267
-// -> 488 us (169 -> 49 FP64 warp instructions per 32 particles), 1000 x 700
+// Measured (EXACT64, one time step, by events on 16-row tiles): 2048^2 composite on
+// the tile kernel 1,267 -> 488 us (169 -> 49 FP64 warp instructions per 32 particles;
+// 481 on 8-row tiles, tile2d.cu; single launches under ncu 1,492 -> 476), 1000 x 700
 // 236 -> 93 us, the 90 x 81 x 77 foam on the spring lists 151 -> 70 us (30 -> 6
 // per 32 springs). What stays on the FP64 pipe: the vector's subtractions, the
 // sum of the squares, r - r0, the gather and the integration.
