@@ -81,7 +81,9 @@ inline double max_critical_length(const std::vector<SpringType> &types)
 //     of a soft phase lose a factor of its contrast: 3e-12 k r0 at 1,000, single
 //     precision at 1e6.
 // Intact springs with |k (1 - r0/r)| up to cmax (df_cmax) stay in the exact range;
-// a particle with one above it is summed with error terms, with no loss.
+// a particle with one above it is summed with error terms, with no loss. (A test of
+// the multiples themselves needs no bound on the springs' lengths and reaches a
+// little further, but costs every spring more: 2048^2 step 117.0 -> 119.7 us.)
 struct DfSplit {
     double unit = 0x1p-21, cmax = 0.0;
 };
