@@ -217,14 +217,12 @@ __device__ __forceinline__ bool spring3(const Tile3Args &A, const long long *dl,
 // partial sum is exact, see DfSum), and with them from there on. (Running all 18
 // springs again with error terms instead took the 256^3 foam from 754 to 970 us
 // a step at 10% compression, 797 this way.)
-template <int PREC, bool TEST>
+template <int PREC>
 __device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, const TypeDF *sdf, const int *soff,
                                             int ep, int pp, uint16_t mk, const long long (&xp)[3], DfSumCareful (&F)[3],
                                             uint16_t &newb)
 {
-    // F32's forces are plain floats, and without a break test springs longer than the
-    // range allows for may be there: always with error terms
-    bool big = PREC != LSM_PREC_DF || !TEST;
+    bool big = PREC != LSM_PREC_DF;  // F32's forces are plain floats: always with error terms
 #pragma unroll 1
     for (int s = 0; s < 9; s++) {
         const int o = soff[s], ei = ep - o, eo = ep + o, sh = A.ssh[s] - 1;
@@ -261,7 +259,7 @@ __device__ __forceinline__ void tile3_pairs(const Tile3Args &A, const Smem3 &S, 
                 f[c][1] = ff{-ff3[c][1], 0.0f};
             }
         }
-        if (TEST && brk[1]) newb |= (uint16_t)(1u << s);
+        if (brk[1]) newb |= (uint16_t)(1u << s);
         if (big) {
 #pragma unroll
             for (int c = 0; c < 3; c++) {
@@ -390,12 +388,14 @@ k_tile3d(Tile3Args A)
 #pragma unroll
         for (int c = 0; c < 3; c++) F3[c].hs = F3[c].el = 0.0f;
         uint16_t newb = 0;
-        if constexpr (!SAMPLE) {
+        if constexpr (MODE == T_STEP && !SAMPLE) {
             // a slot's incoming (source p - o_s) and outgoing (target p + o_s)
             // springs side by side on packed instructions
-            tile3_pairs<PREC, MODE == T_STEP>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb);
+            tile3_pairs<PREC>(A, S, sdf, soff, ep, pp, mk, xp, F3, newb);
         } else {
-            // the same springs in the same order, one at a time
+            // the same springs in the same order, one at a time (initial accelerations
+            // too, which have no break test: the pairs' springs beyond their critical
+            // length give no force)
 #pragma unroll 1
             for (int s = 0; s < 9; s++) {
                 const int sh = A.ssh[s] - 1, ei = ep - soff[s], eo = ep + soff[s];
